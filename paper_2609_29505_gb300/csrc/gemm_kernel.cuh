@@ -932,70 +932,101 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
   const CtaWork w = cta_work(a, num_tiles, blockIdx.x, gridDim.x);
 
   if (warp == 0) {
-    if (lane == 0) {
-      int it = 0;
-      for (int u = 0; u < w.n_units; ++u) {
-        int tile, k0, k1;
-        unit_at(a, w, u, tile, k0, k1);
-        int m_blk, n_blk;
-        tile_coords(a, tile, m_blk, n_blk);
-        const int rb0 = a.gated ? n_blk * 128 : n_blk * kBN;
-        const int rb1 = a.gated ? a.N + n_blk * 128 : rb0 + 128;  // BN = 256 only
-        bool ok = true;
-        for (int kb = k0; kb < k1; ++kb, ++it) {
-          const int s = it % kStages;
-          const uint32_t ph = (it / kStages) & 1;
-          if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, a.status, 1)) {
-            ok = false;
-            break;
-          }
-          uint8_t* st = tiles + s * kStageBytes;
-          mbar_arrive_expect_tx(&full[s], kStageBytes);
-          tma_load_2d(st, &a.tmap_a, &full[s], kb * kBK, m_blk * kBM);
-          tma_load_2d(st + kTileA, &a.tmap_b, &full[s], kb * kBK, rb0);
-          if (kBN == 256) tma_load_2d(st + kTileA + kTileBHalf, &a.tmap_b, &full[s], kb * kBK, rb1);
+    const bool lead = elect_one();
+    const uint32_t tiles0 = smem_u32(tiles), full0 = smem_u32(full), empty0 = smem_u32(empty);
+    uint32_t st = 0, ph = 1;  // ring slot and the parity of its last release
+    int it = 0;
+    bool ok = true;
+    for (int u = 0; u < w.n_units && ok; ++u) {
+      int tile, k0, k1;
+      unit_at(a, w, u, tile, k0, k1);
+      int m_blk, n_blk;
+      tile_coords(a, tile, m_blk, n_blk);
+      const int row_a = m_blk * kBM;
+      const int rb0 = a.gated ? n_blk * 128 : n_blk * kBN;
+      const int rb1 = a.gated ? a.N + n_blk * 128 : rb0 + 128;  // BN = 256 only
+      for (int kb = k0; kb < k1; ++kb, ++it) {
+        const uint32_t bar = full0 + 8 * st;
+        if (!mbar_wait_warp(empty0 + 8 * st, ph, abort_flag, a.status, 1)) {
+          ok = false;
+          break;
         }
-        if (!ok) break;
-      }
-      if (*abort_flag) {
-        // wait for the loads still in flight (the latest issue of each stage)
-        for (int i = (it > kStages ? it - kStages : 0); i < it; ++i)
-          drain_wait(&full[i % kStages], (i / kStages) & 1);
+        if (lead) {
+          const uint32_t dst = tiles0 + st * kStageBytes;
+          mbar_arrive_expect_tx_at(bar, kStageBytes);
+          tma_load_2d_at(dst, &a.tmap_a, bar, kb * kBK, row_a);
+          tma_load_2d_at(dst + kTileA, &a.tmap_b, bar, kb * kBK, rb0);
+          if (kBN == 256) tma_load_2d_at(dst + kTileA + kTileBHalf, &a.tmap_b, bar, kb * kBK, rb1);
+        }
+        if (++st == kStages) {
+          st = 0;
+          ph ^= 1;
+        }
       }
     }
+    if (lead && *abort_flag) {
+      // wait for the loads still in flight (the latest issue of each stage)
+      for (int i = (it > kStages ? it - kStages : 0); i < it; ++i)
+        drain_wait(&full[i % kStages], (i / kStages) & 1);
+    }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_f16(kBM, kBN);
-      int it = 0;
-      bool ok = true;
-      for (int u = 0; u < w.n_units && ok; ++u) {
-        int tile, k0, k1;
-        unit_at(a, w, u, tile, k0, k1);
-        const int acc = u & 1;
-        const uint32_t aph = (u >> 1) & 1;
-        if (!mbar_wait(&tempty[acc], aph ^ 1u, abort_flag, a.status, 2)) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * kBN;
-        for (int kb = k0; kb < k1; ++kb, ++it) {
-          const int s = it % kStages;
-          const uint32_t ph = (it / kStages) & 1;
-          if (!mbar_wait(&full[s], ph, abort_flag, a.status, 3)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a_addr = smem_u32(tiles + s * kStageBytes);
-          const uint32_t b_addr = a_addr + kTileA;
-#pragma unroll
-          for (int k = 0; k < kBK / 16; ++k) {
-            umma_f16(d_tmem, operand_desc<BK>(a_addr + 32 * k), operand_desc<BK>(b_addr + 32 * k),
-                      idesc, (kb != k0 || k != 0) ? 1u : 0u);
-          }
-          umma_commit(&empty[s]);
+    // The whole warp runs the loop and one elected lane issues.  A K-block is 256 (BN 128) to
+    // 512 (BN 256) tensor-core clocks, and one thread spends several clocks on every dependent
+    // instruction, so the loop is kept short: ring slot and descriptors advance by additions
+    // on warp-uniform values, and the next K-block's barrier is tested in between the MMAs of
+    // this one.  (A single divergent thread that derived them from the iteration number took
+    // 566 clocks per K-block at either width, which bounded every GEMM; this form takes 309
+    // and 513.)
+    const bool lead = elect_one();
+    constexpr uint32_t idesc = umma_idesc_f16(kBM, kBN);
+    const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty);
+    const uint64_t desc_a0 = operand_desc<BK>(smem_u32(tiles)), desc_b0 = operand_desc<BK>(smem_u32(tiles) + kTileA);
+    uint64_t da = desc_a0, db = desc_b0;
+    uint32_t st = 0, ph = 0;
+    bool ok = true, ready = false;
+    for (int u = 0; u < w.n_units && ok; ++u) {
+      int tile, k0, k1;
+      unit_at(a, w, u, tile, k0, k1);
+      const int acc = u & 1;
+      const uint32_t aph = (u >> 1) & 1;
+      if (!mbar_wait_warp(smem_u32(&tempty[acc]), aph ^ 1u, abort_flag, a.status, 2)) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + acc * kBN;
+      uint32_t accumulate = 0;
+      for (int kb = k0; kb < k1; ++kb) {
+        if (!ready && !mbar_wait_warp(full0 + 8 * st, ph, abort_flag, a.status, 3)) {
+          ok = false;
+          break;
         }
-        if (!ok) break;
-        umma_commit(&tfull[acc]);
+        tc_fence_after();
+        const uint32_t bar = empty0 + 8 * st;
+        if (lead) {
+          // K slice k of a row block starts 32 k bytes (2 k descriptor units) further
+          umma_f16(d_tmem, da, db, idesc, accumulate);
+          if (kBK == 64) umma_f16(d_tmem, da + 2, db + 2, idesc, 1u);
+        }
+        accumulate = 1;
+        const uint64_t ca = da, cb = db;
+        da += kStageBytes >> 4;
+        db += kStageBytes >> 4;
+        if (++st == kStages) {
+          st = 0;
+          ph ^= 1;
+          da = desc_a0;
+          db = desc_b0;
+        }
+        ready = mbar_test_warp(full0 + 8 * st, ph);
+        if (lead) {
+          constexpr int kRest = kBK == 64 ? 2 : 1;
+#pragma unroll
+          for (int k = kRest; k < kBK / 16; ++k) umma_f16(d_tmem, ca + 2 * k, cb + 2 * k, idesc, 1u);
+          umma_commit_at(bar);
+        }
       }
+      if (!ok) break;
+      if (lead) umma_commit_at(smem_u32(&tfull[acc]));
+    }
+    if (lead) {
       // every MMA issued by this thread has finished once `drain` completes
       umma_commit(drain);
       drain_wait(drain, 0);
