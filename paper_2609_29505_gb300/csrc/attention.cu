@@ -638,94 +638,103 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      const int col0 = h * a.head_stride;
-      // one 128-row operand tile: its 64-column atoms, then (d_h 72) its 16-column atom
-      auto load_tile = [&](uint8_t* dst, const CUtensorMap* m64, const CUtensorMap* m16, uint64_t* bar,
-                           int row) {
-        for (int at = 0; at < L::kA64; ++at) tma_load_2d(dst + at * kAtom, m64, bar, col0 + at * 64, row);
-        if (L::kPad) tma_load_2d(dst + L::kA64 * kAtom, m16, bar, col0 + 64, row);
-      };
-      mbar_arrive_expect_tx(q_full, (two ? 2 : 1) * L::kTile);
+    const bool lead = elect_one();
+    const uint32_t sm0 = smem_u32(sm), kv_full0 = smem_u32(kv_full), kv_empty0 = smem_u32(kv_empty);
+    const int col0 = h * a.head_stride;
+    // one 128-row operand tile: its 64-column atoms, then (d_h 72) its 16-column atom
+    auto load_tile = [&](uint32_t dst, const CUtensorMap* m64, const CUtensorMap* m16, uint32_t bar, int row) {
+      for (int at = 0; at < L::kA64; ++at) tma_load_2d_at(dst + at * kAtom, m64, bar, col0 + at * 64, row);
+      if (L::kPad) tma_load_2d_at(dst + L::kA64 * kAtom, m16, bar, col0 + 64, row);
+    };
+    if (lead) {
+      const uint32_t bar = smem_u32(q_full);
+      mbar_arrive_expect_tx_at(bar, (two ? 2 : 1) * L::kTile);
       for (int t = 0; t < (two ? 2 : 1); ++t)
-        load_tile(sm + L::kQ + t * L::kTile, &a.tmap_q, &a.tmap_q16, q_full, b * a.n_q + (2 * qt + t) * kTcBQ);
-      int j = 0;
-      for (; j < nt; ++j) {
-        const int s = j & 1;
-        if (!mbar_wait(&kv_empty[s], ((j >> 1) & 1) ^ 1u, abort_flag, a.status, 21)) break;
-        uint8_t* st = sm + L::kKV + s * L::kStage;
-        mbar_arrive_expect_tx(&kv_full[s], 2 * L::kTile);
+        load_tile(sm0 + L::kQ + t * L::kTile, &a.tmap_q, &a.tmap_q16, bar, b * a.n_q + (2 * qt + t) * kTcBQ);
+    }
+    int j = 0;
+    for (; j < nt; ++j) {
+      const int s = j & 1;
+      if (!mbar_wait_warp(kv_empty0 + 8 * s, ((j >> 1) & 1) ^ 1u, abort_flag, a.status, 21)) break;
+      if (lead) {
+        const uint32_t st = sm0 + L::kKV + s * L::kStage, bar = kv_full0 + 8 * s;
+        mbar_arrive_expect_tx_at(bar, 2 * L::kTile);
         const int row = b * a.n_kv + j * kTcBK;
-        load_tile(st, &a.tmap_k, &a.tmap_k16, &kv_full[s], row);
-        load_tile(st + L::kTile, &a.tmap_v, &a.tmap_v16, &kv_full[s], row);
-      }
-      if (*abort_flag) {
-        drain_bar(q_full, 0);
-        for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) drain_bar(&kv_full[i & 1], (i >> 1) & 1);
+        load_tile(st, &a.tmap_k, &a.tmap_k16, bar, row);
+        load_tile(st + L::kTile, &a.tmap_v, &a.tmap_v16, bar, row);
       }
     }
+    if (lead && *abort_flag) {
+      drain_bar(q_full, 0);
+      for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) drain_bar(&kv_full[i & 1], (i >> 1) & 1);
+    }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc_qk = umma_idesc_f16(kTcBQ, kTcBK);
-      const uint32_t idesc_pv = umma_idesc_f16_bmn(kTcBQ, 64 * L::kA64);
-      const uint32_t idesc_pv16 = umma_idesc_f16_bmn(kTcBQ, 16);
-      bool ok = mbar_wait(q_full, 0, abort_flag, a.status, 22);
-      auto issue_qk = [&](int t, int j) {
-        const int s = j & 1;
-        const uint32_t qa = smem_u32(sm + L::kQ + t * L::kTile);
-        const uint32_t ka = smem_u32(sm + L::kKV + s * L::kStage);
+    // The whole warp runs the loop, one elected lane issues, and every operand of an MMA is a
+    // warp-uniform base plus a constant: a single divergent thread that built each descriptor
+    // took about 140 clocks per MMA, twice what a 128 x 128 x 16 MMA takes to run.
+    const bool lead = elect_one();
+    constexpr uint32_t idesc_qk = umma_idesc_f16(kTcBQ, kTcBK);
+    constexpr uint32_t idesc_pv = umma_idesc_f16_bmn(kTcBQ, 64 * L::kA64);
+    constexpr uint32_t idesc_pv16 = umma_idesc_f16_bmn(kTcBQ, 16);
+    const uint32_t sm0 = smem_u32(sm), kv_full0 = smem_u32(kv_full), kv_empty0 = smem_u32(kv_empty);
+    const uint32_t s_full0 = smem_u32(s_full), p_full0 = smem_u32(p_full), o_done0 = smem_u32(o_done);
+    const uint64_t dq = smem_desc_sw128(sm0 + L::kQ), dk = smem_desc_sw128(sm0 + L::kKV);
+    const uint64_t dv = smem_desc_sw128_mn(sm0 + L::kKV + L::kTile, kAtom, 1024);
+    const uint64_t dq16 = smem_desc_sw32(sm0 + L::kQ + L::kA64 * kAtom);
+    const uint64_t dk16 = smem_desc_sw32(sm0 + L::kKV + L::kA64 * kAtom);
+    const uint64_t dv16 = smem_desc_sw32_mn(sm0 + L::kKV + L::kTile + L::kA64 * kAtom, kAtom32, 256);
+    constexpr uint64_t kTileU = L::kTile >> 4, kStageU = L::kStage >> 4;  // in descriptor units of 16 bytes
+    bool ok = mbar_wait_warp(smem_u32(q_full), 0, abort_flag, a.status, 22);
+    auto issue_qk = [&](int t, int s) {
+      if (!lead) return;
+      const uint32_t d = tmem + L::kTmemS + t * kTcBK;
+      const uint64_t qa = dq + t * kTileU, ka = dk + s * kStageU;
 #pragma unroll
-        for (int ks = 0; ks < 4 * L::kA64; ++ks) {
-          const uint32_t off = (ks >> 2) * kAtom + (ks & 3) * 32;
-          umma_f16(tmem + L::kTmemS + t * kTcBK, smem_desc_sw128(qa + off), smem_desc_sw128(ka + off),
-                   idesc_qk, ks > 0 ? 1u : 0u);
-        }
-        if (L::kPad) {  // head columns 64..79 (Q's 72..79 are zero)
-          const uint32_t off = L::kA64 * kAtom;
-          umma_f16(tmem + L::kTmemS + t * kTcBK, smem_desc_sw32(qa + off), smem_desc_sw32(ka + off),
-                   idesc_qk, 1u);
-        }
-        umma_commit(&s_full[t]);
-      };
-      auto issue_pv = [&](int t, int j) {
-        const int s = j & 1;
-        const uint32_t va = smem_u32(sm + L::kKV + s * L::kStage + L::kTile);
+      for (int ks = 0; ks < 4 * L::kA64; ++ks) {
+        const uint64_t off = ((ks >> 2) * kAtom + (ks & 3) * 32) >> 4;
+        umma_f16(d, qa + off, ka + off, idesc_qk, ks > 0 ? 1u : 0u);
+      }
+      if (L::kPad)  // head columns 64..79 (Q's 72..79 are zero)
+        umma_f16(d, dq16 + t * kTileU, dk16 + s * kStageU, idesc_qk, 1u);
+      umma_commit_at(s_full0 + 8 * t);
+    };
+    auto issue_pv = [&](int t, int s, uint32_t accumulate) {
+      if (!lead) return;
+      const uint32_t pa = tmem + L::kTmemS + t * kTcBK, d = tmem + L::kTmemO + t * L::kDP;
+      const uint64_t va = dv + s * kStageU, va16 = dv16 + s * kStageU;
 #pragma unroll
-        for (int ks = 0; ks < kTcBK / 16; ++ks) {
-          const uint64_t bd = smem_desc_sw128_mn(va + ks * 2048, kAtom, 1024);
-          const uint32_t pa = tmem + L::kTmemS + t * kTcBK + 8 * ks;
-          umma_f16_ts(tmem + L::kTmemO + t * L::kDP, pa, bd, idesc_pv, (j > 0 || ks > 0) ? 1u : 0u);
-          if (L::kPad) {  // O columns 64..79 from the 16-column V atom (8-key-row groups 256 B apart)
-            const uint64_t bd16 = smem_desc_sw32_mn(va + L::kA64 * kAtom + ks * 512, kAtom32, 256);
-            umma_f16_ts(tmem + L::kTmemO + t * L::kDP + 64 * L::kA64, pa, bd16, idesc_pv16,
-                        (j > 0 || ks > 0) ? 1u : 0u);
-          }
-        }
-        umma_commit(&o_done[t]);
-      };
-      if (ok && (ok = mbar_wait(&kv_full[0], 0, abort_flag, a.status, 23))) {
-        tc_fence_after();
-        issue_qk(0, 0);
-        if (two) issue_qk(1, 0);
+      for (int ks = 0; ks < kTcBK / 16; ++ks) {
+        umma_f16_ts(d, pa + 8 * ks, va + ks * (2048 >> 4), idesc_pv, ks > 0 ? 1u : accumulate);
+        if (L::kPad)  // O columns 64..79 from the 16-column V atom (8-key-row groups 256 B apart)
+          umma_f16_ts(d + 64 * L::kA64, pa + 8 * ks, va16 + ks * (512 >> 4), idesc_pv16, ks > 0 ? 1u : accumulate);
       }
-      for (int j = 0; j < nt && ok; ++j) {
-        const uint32_t ph = j & 1;
-        if (!(ok = mbar_wait(&p_full[0], ph, abort_flag, a.status, 24))) break;
+      umma_commit_at(o_done0 + 8 * t);
+    };
+    if (ok && (ok = mbar_wait_warp(kv_full0, 0, abort_flag, a.status, 23))) {
+      tc_fence_after();
+      issue_qk(0, 0);
+      if (two) issue_qk(1, 0);
+    }
+    for (int j = 0; j < nt && ok; ++j) {
+      const int s = j & 1;
+      const uint32_t ph = j & 1, acc = j > 0 ? 1u : 0u;
+      if (!(ok = mbar_wait_warp(p_full0, ph, abort_flag, a.status, 24))) break;
+      tc_fence_after();
+      issue_pv(0, s, acc);
+      if (j + 1 < nt) {
+        if (!(ok = mbar_wait_warp(kv_full0 + 8 * (s ^ 1), ((j + 1) >> 1) & 1, abort_flag, a.status, 25))) break;
         tc_fence_after();
-        issue_pv(0, j);
-        if (j + 1 < nt) {
-          if (!(ok = mbar_wait(&kv_full[(j + 1) & 1], ((j + 1) >> 1) & 1, abort_flag, a.status, 25))) break;
-          tc_fence_after();
-          issue_qk(0, j + 1);
-        }
-        if (two) {
-          if (!(ok = mbar_wait(&p_full[1], ph, abort_flag, a.status, 26))) break;
-          tc_fence_after();
-          issue_pv(1, j);
-        }
-        umma_commit(&kv_empty[j & 1]);
-        if (two && j + 1 < nt) issue_qk(1, j + 1);
+        issue_qk(0, s ^ 1);
       }
+      if (two) {
+        if (!(ok = mbar_wait_warp(p_full0 + 8, ph, abort_flag, a.status, 26))) break;
+        tc_fence_after();
+        issue_pv(1, s, acc);
+      }
+      if (lead) umma_commit_at(kv_empty0 + 8 * s);
+      if (two && j + 1 < nt) issue_qk(1, s ^ 1);
+    }
+    if (lead) {
       umma_commit(drain);
       drain_bar(drain, 0);
     }
@@ -740,7 +749,7 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
     bool ok = t == 0 || two;  // the warpgroup of an empty second tile has nothing to do
     uint32_t r[kTcBK];
     for (int j = 0; j < nt && ok; ++j) {
-      if (!(ok = warp_wait_bar(&s_full[t], j & 1, abort_flag, a.status, 27))) break;
+      if (!(ok = mbar_wait_warp(smem_u32(&s_full[t]), j & 1, abort_flag, a.status, 27))) break;
       tc_fence_after();
       const int kb = j * kTcBK;
       const int nvalid = min(a.n_kv - kb, kTcBK);  // keys of this tile (the rest are masked)
@@ -766,7 +775,7 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
         m2 = mt;
       } else if (__any_sync(0xffffffffu, mt > m2 + kRescaleLog2)) {
         // warp-uniform (the TMEM accesses are .sync.aligned); O_t must hold PV_t(j-1)
-        if (!(ok = warp_wait_bar(&o_done[t], (j - 1) & 1, abort_flag, a.status, 28))) break;
+        if (!(ok = mbar_wait_warp(smem_u32(&o_done[t]), (j - 1) & 1, abort_flag, a.status, 28))) break;
         tc_fence_after();
         const float mnew = fmaxf(m2, mt);
         const float corr = exp2f(m2 - mnew);
@@ -807,7 +816,7 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
       __syncwarp();
       if (lane == 0) mbar_arrive(&p_full[t]);
     }
-    if (ok && warp_wait_bar(&o_done[t], (nt - 1) & 1, abort_flag, a.status, 29)) {
+    if (ok && mbar_wait_warp(smem_u32(&o_done[t]), (nt - 1) & 1, abort_flag, a.status, 29)) {
       tc_fence_after();
       const float inv = 1.f / l;
       const int qrow = (2 * qt + t) * kTcBQ + row;
