@@ -73,12 +73,47 @@ __device__ __forceinline__ void unpack_f16x8(const uint4& u, float* f) {
   }
 }
 
+// max(|a|, |b|, |c|), NaN if any is NaN (one instruction on sm_100 and later)
+__device__ __forceinline__ float absmax3_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
+// Eight values as pack_f16x2 rounds and clamps them.  The clamp is rare, so the eight are
+// checked together (four instructions instead of four per value) and rounded as they are
+// unless one of them is out of range: packing was most of the instructions of an fp16
+// epilogue.
 __device__ __forceinline__ uint4 pack_f16x8(const float* f) {
+  const float m = absmax3_nan(absmax3_nan(f[0], f[1], f[2]), absmax3_nan(f[3], f[4], f[5]), absmax3_nan(f[6], f[7], 0.f));
   uint4 u;
+  if (m <= 65504.f) {
+    const __half2 h0 = __floats2half2_rn(f[0], f[1]), h1 = __floats2half2_rn(f[2], f[3]);
+    const __half2 h2 = __floats2half2_rn(f[4], f[5]), h3 = __floats2half2_rn(f[6], f[7]);
+    u.x = *reinterpret_cast<const uint32_t*>(&h0);
+    u.y = *reinterpret_cast<const uint32_t*>(&h1);
+    u.z = *reinterpret_cast<const uint32_t*>(&h2);
+    u.w = *reinterpret_cast<const uint32_t*>(&h3);
+    return u;
+  }
   u.x = pack_f16x2(f[0], f[1]);
   u.y = pack_f16x2(f[2], f[3]);
   u.z = pack_f16x2(f[4], f[5]);
   u.w = pack_f16x2(f[6], f[7]);
+  return u;
+}
+
+__device__ __forceinline__ uint2 pack_f16x4(float4 f) {
+  const float m = absmax3_nan(absmax3_nan(f.x, f.y, f.z), f.w, 0.f);
+  uint2 u;
+  if (m <= 65504.f) {
+    const __half2 h0 = __floats2half2_rn(f.x, f.y), h1 = __floats2half2_rn(f.z, f.w);
+    u.x = *reinterpret_cast<const uint32_t*>(&h0);
+    u.y = *reinterpret_cast<const uint32_t*>(&h1);
+    return u;
+  }
+  u.x = pack_f16x2(f.x, f.y);
+  u.y = pack_f16x2(f.z, f.w);
   return u;
 }
 

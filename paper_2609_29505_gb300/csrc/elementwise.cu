@@ -94,12 +94,7 @@ __device__ __forceinline__ float4 norm_affine_s(const NormParams& p, int i, floa
   return make_float4(y[0], y[1], y[2], y[3]);
 }
 
-__device__ __forceinline__ void store_f16x4(f16* p, float4 v) {
-  uint2 u;
-  u.x = pack_f16x2(v.x, v.y);
-  u.y = pack_f16x2(v.z, v.w);
-  *reinterpret_cast<uint2*>(p) = u;
-}
+__device__ __forceinline__ void store_f16x4(f16* p, float4 v) { *reinterpret_cast<uint2*>(p) = pack_f16x4(v); }
 
 __global__ void __launch_bounds__(kNormThreads) norm_kernel(const NormParams p) {
   __shared__ float red[kNormThreads / 32];
@@ -705,10 +700,7 @@ __global__ void pack_f16_kernel(f16* dst, int ld_dst, int col0, const float* h, 
     const int64_t r = e / d;
     const int c = static_cast<int>(e % d);
     const float4 v = reinterpret_cast<const float4*>(h)[i];
-    uint2 u;
-    u.x = pack_f16x2(v.x, v.y);
-    u.y = pack_f16x2(v.z, v.w);
-    *reinterpret_cast<uint2*>(dst + r * ld_dst + col0 + c) = u;
+    store_f16x4(dst + r * ld_dst + col0 + c, v);
   }
 }
 

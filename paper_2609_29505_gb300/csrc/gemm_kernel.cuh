@@ -29,6 +29,7 @@
 #pragma once
 
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -336,82 +337,75 @@ __device__ __forceinline__ void emit_stats(const EpiParams& e, int row, int slot
 
 // Residual epilogue through this warp's 4 KB staging buffer `stg` (32 rows x 8 float4,
 // 16-byte chunk j of row r at r * 8 + (j ^ (r & 7)), so that both access patterns below are
-// free of bank conflicts).  Per 32-column chunk: the warp loads its 32 rows of h coalesced
-// (8 lanes per 128-byte row segment), each thread adds its row's accumulator (times the
-// AdaLN gate) in shared memory, and the warp stores h and the fp16 cache coalesced.  With
-// one thread per row the same accesses touch 32 rows per instruction, which made the
-// epilogue of a short-K projection take longer than its main loop.
-template <class Src>
+// free of bank conflicts).  Per 32-column chunk each thread puts its row's accumulator in
+// shared memory, and the warp then reads, updates and stores h and the fp16 cache with 8 lanes
+// per 128-byte row segment (with one thread per row the same accesses touch 32 rows per
+// instruction).  h does not depend on the accumulator: load_h_chunk fetches the first chunk
+// before the wait for it, and every further chunk while the one before is added, so that no
+// global load latency is left between the last MMA and the last store.
+__device__ __forceinline__ void load_h_chunk(const TcArgs& a, int row0, int col0, float4* hv) {
+  const int lane = threadIdx.x & 31;
+  const int lr = lane >> 3, col = col0 + 4 * (lane & 7);
+#pragma unroll
+  for (int it = 0; it < 8; ++it) {
+    const int r = row0 + it * 4 + lr;
+    hv[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < a.M && col < a.N)  // N % 8 == 0
+      hv[it] = *reinterpret_cast<const float4*>(a.epi.h + static_cast<int64_t>(r) * a.epi.ldh + col);
+  }
+}
+
+// kAhead: hv holds the first chunk of h (otherwise, for stream-K partial sums, whose source
+// needs the registers, each chunk is loaded where it is used).
+template <bool kAhead, class Src>
 __device__ __forceinline__ void delta_staged(const TcArgs& a, int row, int n0, const Src& src, int cb, int ce,
-                                             float4* stg) {
+                                             float4* stg, float4* hv) {
   const EpiParams& e = a.epi;
   const int lane = threadIdx.x & 31;
   const int row0 = row - lane;  // the warp's first row
   const int lr = lane >> 3, lc = lane & 7;
-  const bool row_ok = row < a.M;
-  const float* grow =
-      e.gate ? e.gate + static_cast<int64_t>(row_ok ? row / e.rows_per_batch : 0) * e.ld_gate + n0 : nullptr;
+  // AdaLN gate: one vector per chunk where the warp's 32 rows belong to one sample
+  const int smp = e.gate ? row0 / e.rows_per_batch : 0;
+  const bool one_smp = e.gate && (row0 + 31) / e.rows_per_batch == smp;
 #pragma unroll 1
   for (int c = cb; c < ce; c += 32) {
-    const int col0 = n0 + c;
+    const int col0 = n0 + c, col = col0 + 4 * lc;
     if (col0 >= a.N) break;
-    const bool c_ok = col0 + 4 * lc < a.N;  // this lane's float4 in the coalesced phases (N % 8 == 0)
+    const bool c_ok = col < a.N;  // this lane's float4 in the coalesced phase (N % 8 == 0)
+    float4 gv = make_float4(1.f, 1.f, 1.f, 1.f);
+    if (one_smp && c_ok && row0 < a.M)
+      gv = *reinterpret_cast<const float4*>(e.gate + static_cast<int64_t>(smp) * e.ld_gate + col);
     {
-      float4 hv[8];
+      float x[16], y[16];
+      src.load2(c, c + 16, x, y);
 #pragma unroll
-      for (int it = 0; it < 8; ++it) {
-        const int r = row0 + it * 4 + lr;
-        hv[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < a.M && c_ok)
-          hv[it] = *reinterpret_cast<const float4*>(e.h + static_cast<int64_t>(r) * e.ldh + col0 + 4 * lc);
-      }
-#pragma unroll
-      for (int it = 0; it < 8; ++it) {
-        const int r = it * 4 + lr;
-        stg[r * 8 + (lc ^ (r & 7))] = hv[it];
+      for (int j = 0; j < 8; ++j) {
+        const float* v = j < 4 ? x + 4 * j : y + 4 * (j - 4);
+        stg[lane * 8 + (j ^ (lane & 7))] = make_float4(v[0], v[1], v[2], v[3]);
       }
     }
-    __syncwarp();
-    float x[16], y[16];
-    src.load2(c, c + 16, x, y);
-    if (grow) {  // columns past N (the tile's edge) read the row's last four, never stored
+    float4 h4[8];
+    if constexpr (kAhead) {
 #pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        const float4 gv = *reinterpret_cast<const float4*>(grow + min(c + 4 * g, a.N - n0 - 4));
-        float* v = g < 4 ? x + 4 * g : y + 4 * (g - 4);
-        v[0] *= gv.x; v[1] *= gv.y; v[2] *= gv.z; v[3] *= gv.w;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float* v = j < 4 ? x + 4 * j : y + 4 * (j - 4);
-      float4& hs = stg[lane * 8 + (j ^ (lane & 7))];
-      float4 h4 = hs;
-      h4.x += v[0]; h4.y += v[1]; h4.z += v[2]; h4.w += v[3];
-      hs = h4;
+      for (int it = 0; it < 8; ++it) h4[it] = hv[it];
+      if (c + 32 < ce) load_h_chunk(a, row0, col0 + 32, hv);
+    } else {
+      load_h_chunk(a, row0, col0, h4);
     }
     __syncwarp();
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
-      const int r = it * 4 + lr;
-      if (row0 + r < a.M && c_ok)
-        *reinterpret_cast<float4*>(e.h + static_cast<int64_t>(row0 + r) * e.ldh + col0 + 4 * lc) =
-            stg[r * 8 + (lc ^ (r & 7))];
-    }
-    if (e.cache) {
-      __syncwarp();
-      uint4* su = reinterpret_cast<uint4*>(stg);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) su[lane * 8 + (j ^ (lane & 7))] = pack_f16x8(j < 2 ? x + 8 * j : y + 8 * (j - 2));
-      __syncwarp();
-      const int lr4 = lane >> 2, lc4 = lane & 3;
-      const bool c8_ok = col0 + 8 * lc4 < a.N;
-#pragma unroll
-      for (int it = 0; it < 4; ++it) {
-        const int r = it * 8 + lr4;
-        if (row0 + r < a.M && c8_ok)
-          *reinterpret_cast<uint4*>(e.cache + static_cast<int64_t>(row0 + r) * e.ld_cache + col0 + 8 * lc4) =
-              su[r * 8 + (lc4 ^ (r & 7))];
+      const int r = it * 4 + lr, gr = row0 + r;
+      float4 v = stg[r * 8 + (lc ^ (r & 7))];
+      if (gr < a.M && c_ok) {
+        if (e.gate) {
+          if (!one_smp)
+            gv = *reinterpret_cast<const float4*>(e.gate + static_cast<int64_t>(gr / e.rows_per_batch) * e.ld_gate + col);
+          v.x *= gv.x; v.y *= gv.y; v.z *= gv.z; v.w *= gv.w;
+        }
+        *reinterpret_cast<float4*>(e.h + static_cast<int64_t>(gr) * e.ldh + col) =
+            make_float4(h4[it].x + v.x, h4[it].y + v.y, h4[it].z + v.z, h4[it].w + v.w);
+        if (e.cache) *reinterpret_cast<uint2*>(e.cache + static_cast<int64_t>(gr) * e.ld_cache + col) = pack_f16x4(v);
       }
     }
     __syncwarp();  // the next chunk overwrites the staging buffer
@@ -479,7 +473,7 @@ __device__ __forceinline__ void stage_flush_f32(const EpiParams& e, void* out, i
 template <int BN, bool kFastRope, int FEAT, class Src>
 __device__ __forceinline__ void epilogue_tile(const TcArgs& a, void* out, int row, int n_blk,
                                               const Src& src, int cb, int ce, int part, int halves,
-                                              float4* stg) {
+                                              float4* stg, float4* hv) {
   constexpr int kBN = BN;
   constexpr bool kH16 = FEAT == kFeatH16;
   // compile-time pruning of paths a feature set never takes (gemm_plan enforces it): a
@@ -617,7 +611,7 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& a, void* out, int ro
   if (!kNormFeat && e.kind == SGD_EPI_DELTA) {
     if constexpr (!kH16 && !kFastRope) {  // 8-warp kernels (the 4-warp RoPE kernel has no registers to spare)
       if (stg != nullptr) {
-        delta_staged(a, row, n0, src, cb, ce, stg);
+        delta_staged<std::is_same<Src, TmemSrc>::value>(a, row, n0, src, cb, ce, stg, hv);
         return;
       }
     }
@@ -1047,6 +1041,8 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
     const int pe = kEpiWarps == 8 ? (part ? kBN : kSplit) : kBN;
     const int total = a.sk_tiles * a.num_k;
     void* out = a.epi.out_slot ? *a.epi.out_slot : a.epi.out;
+    const bool h_ahead = FEAT == kFeatPlain && C::kStaging > 0 && a.epi.kind == SGD_EPI_DELTA;
+    float4 hv[8];  // first 32-column chunk of h (delta_staged)
     for (int u = 0; u < w.n_units; ++u) {
       int tile, k0, k1;
       unit_at(a, w, u, tile, k0, k1);
@@ -1058,12 +1054,13 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kBN;
       if (u >= w.n_sk) {  // data-parallel tile
         prefetch_h_row(a.epi, row, a.M, a.N, n_blk * kBN, cb, ce);
+        if (h_ahead) load_h_chunk(a, row - lane, n_blk * kBN + cb, hv);
         if (FEAT == kFeatH16 && a.epi.stat_cnt) {  // every epilogue thread reaches the barriers
           const bool ok = warp_wait(&tfull[acc], aph, abort_flag, a.status, 4);
           if (ok) {
             tc_fence_after();
             epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, cb, ce,
-                                                     part, kEpiWarps == 8 ? 2 : 1, stg);
+                                                     part, kEpiWarps == 8 ? 2 : 1, stg, hv);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -1074,7 +1071,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
         if (!warp_wait(&tfull[acc], aph, abort_flag, a.status, 4)) break;
         tc_fence_after();
         epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, cb, ce, part,
-                                           kEpiWarps == 8 ? 2 : 1, stg);
+                                           kEpiWarps == 8 ? 2 : 1, stg, hv);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -1085,9 +1082,10 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
       const bool ok = warp_wait(&tfull[acc], aph, abort_flag, a.status, 4);
       if (k0 == 0 && k1 == a.num_k) {  // the whole K range of the tile lies in this CTA's share
         if (ok) {
+          if (h_ahead) load_h_chunk(a, row - lane, n_blk * kBN + cb, hv);
           tc_fence_after();
           epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, cb, ce, part,
-                                           kEpiWarps == 8 ? 2 : 1, stg);
+                                           kEpiWarps == 8 ? 2 : 1, stg, hv);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -1124,7 +1122,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
       if (*last_flag != 0) {
         __threadfence();
         epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, WsSrc<kBN>{slot0, nseg, q * 32 + lane, a.epi.alpha},
-                                           cb, ce, part, kEpiWarps == 8 ? 2 : 1, stg);
+                                           cb, ce, part, kEpiWarps == 8 ? 2 : 1, stg, hv);
         if (threadIdx.x == 64) a.sk_cnt[tile] = 0;
       }
       // the CTA that finished the tile (last_flag is CTA-uniform) draws its row block's ticket
