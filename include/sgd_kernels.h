@@ -102,14 +102,16 @@ SGD_API int sgd_kernel_gemm_stat_slots(int M, int N, int K, const sgd_epilogue_a
 /*
  * C = alpha A B^T.  A fp16 [M, K] (row stride lda elements), B fp16 [N or 2N, K]
  * (row stride ldb).  K, lda, ldb multiples of 8; N multiple of 8; pointers 16-byte
- * aligned.  use_simt = 1 runs the plain SIMT kernel (reference / debugging), 0 the
- * tcgen05 + TMA kernel (M = 128, N = 256, K = 16 instructions, fp32 accumulators in
- * TMEM) with 64-element K-blocks, choosing by itself 128 x 256 or 128 x 128 tiles, 4 or 8
+ * aligned.  use_simt = 1 runs the plain SIMT kernel (reference / debugging), 0 a
+ * tcgen05 + TMA kernel (fp32 accumulators in TMEM) with 64-element K-blocks: where M > 128
+ * and its tiles fit at least as well, the CTA-pair kernel (256 x 128 .. 256 x 256 tiles, M = 256
+ * instructions over two SMs), otherwise the one-CTA kernel (M = 128, N = 256, K = 16
+ * instructions), choosing by itself 128 x 256 or 128 x 128 tiles, 4 or 8
  * epilogue warps, and whether the tiles left over after the last full wave of CTAs are
  * split along K over all SMs ("stream-K": fp32 partial tiles in a workspace, summed in a
  * fixed order by the CTA that finishes a tile last, so results are deterministic); 3 the
  * form of 0 with 32-element K-blocks (64-byte swizzle); 2 and 4 are not defined and are
- * rejected with SGD_ERR_ARG; 5, 6, 7 force 128 x 256 tiles with 4 epilogue warps, 128 x 256 with 8, and
+ * rejected with SGD_ERR_ARG; 3 and 5 to 12 are forms of the one-CTA kernel: 5, 6, 7 force 128 x 256 tiles with 4 epilogue warps, 128 x 256 with 8, and
  * 128 x 128 with 8 and no stream-K (128 x 128 applies to plain, GELU and DELTA epilogues
  * only); 8 is 0 without stream-K, 9 is 0 with stream-K whenever the last wave is partial;
  * 10 forces 128 x 224 tiles (5 pipeline stages, no stream-K; plain, GELU and DELTA only);
@@ -132,8 +134,9 @@ SGD_API int sgd_kernel_gemm(const void* A, int lda, const void* B, int ldb, int 
  * stream-K split keeps its partial tiles and tile tickets: in one fixed array compiled
  * into the library (32 MiB of fp32 partial tiles, then 1024 tickets) instead of a
  * workspace the library allocates.
- * Limit: a problem whose stream-K split needs more than the array holds is rejected
- * with SGD_ERR_SHAPE before anything is launched (variant 8, or sgd_kernel_gemm, runs it).
+ * Limit: a problem whose stream-K split (that of the one-CTA kernel, whichever kernel variant 0
+ * runs) needs more than the array holds is rejected with SGD_ERR_SHAPE before anything is
+ * launched (variant 8, or sgd_kernel_gemm, runs it).
  * The tickets are cleared (cudaMemsetAsync on `stream`) before each stream-K launch; the
  * partial tiles need no clearing (each is written before it is read within one launch).
  * Every call on a device uses the same array: calls that can overlap in time (launched

@@ -799,15 +799,16 @@ struct CtaWork {
   int unit0, unit_step, n_units;
 };
 
-__device__ __forceinline__ CtaWork cta_work(const TcArgs& a, int num_tiles, int unit0, int unit_step) {
+// `worker`: the CTA's (or CTA pair's) index among the sk_ctas of the stream-K split.
+__device__ __forceinline__ CtaWork cta_work(const TcArgs& a, int num_tiles, int unit0, int unit_step, int worker) {
   CtaWork w;
   w.unit0 = unit0;
   w.unit_step = unit_step;
   w.sk_s = w.sk_e = w.t_sk0 = w.n_sk = 0;
-  if (a.sk_tiles > 0 && static_cast<int>(blockIdx.x) < a.sk_ctas) {
+  if (a.sk_tiles > 0 && worker < a.sk_ctas) {
     const int total = a.sk_tiles * a.num_k;
-    w.sk_s = sk_start(blockIdx.x, total, a.sk_ctas);
-    w.sk_e = sk_start(blockIdx.x + 1, total, a.sk_ctas);
+    w.sk_s = sk_start(worker, total, a.sk_ctas);
+    w.sk_e = sk_start(worker + 1, total, a.sk_ctas);
     w.t_sk0 = w.sk_s / a.num_k;
     w.n_sk = (w.sk_e - 1) / a.num_k - w.t_sk0 + 1;
   }
@@ -923,7 +924,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
   const uint32_t tmem_base = *tmem_slot;
   const int num_mu = a.num_m;
   const int num_tiles = num_mu * a.num_n;
-  const CtaWork w = cta_work(a, num_tiles, blockIdx.x, gridDim.x);
+  const CtaWork w = cta_work(a, num_tiles, blockIdx.x, gridDim.x, blockIdx.x);
 
   if (warp == 0) {
     const bool lead = elect_one();

@@ -84,6 +84,8 @@ struct GemmPlan {
   int M = 0, N = 0, K = 0;   // N = output columns
   EpiParams epi{};
   bool simt = false;
+  bool allow_pair = false;   // let gemm_plan choose the CTA-pair kernel (gemm_pair_kernel.cuh)
+  bool pair = false;         // set by gemm_plan: the CTA-pair kernel, 256 x bn tiles
   int bk = 64;               // K elements per stage: 64 (128-byte swizzle) or 32 (64-byte)
   int bn = 0;                // output columns per tile: 256, 128, or 0 = choose by tile count
   int epiw = 0;              // epilogue warps: 4, 8, or 0 = choose by epilogue kind
@@ -106,8 +108,10 @@ int gemm_plan(GemmPlan& p, const char** why);
 cudaError_t gemm_launch(const GemmPlan& p, cudaStream_t s);
 // fp32 elements of stream-K workspace a planned GEMM needs (0: data-parallel only).
 size_t gemm_ws_floats(const GemmPlan& p);
+int gemm_ws_tickets(const GemmPlan& p);  // and int tickets
 // The fixed stream-K scratch of the current device (partials, then tickets) and its
 // capacity; returns 0, or -1 with `why` set when its address cannot be obtained.
+size_t gemm_static_ws_bytes();
 int gemm_static_scratch(float** ws, size_t* ws_floats, int** tickets, int* n_tickets, const char** why);
 int* device_status_ptr();  // device address of the shared status word
 // Accessors of the fp16 clamp flags of every kernel translation unit (registered at load).

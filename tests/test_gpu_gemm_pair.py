@@ -1,0 +1,97 @@
+"""The CTA-pair GEMM (sgd_kernel_gemm variant 0 where M > 128) against the oracle, at one shape
+per tile width and epilogue that the rule picks there, with ragged last tiles in M, N and K.
+Bounds: fp16 results the rounding of the result plus fp32 accumulation; fp32 results
+accumulation alone, 2^-23 x sqrt(K) x the terms' norm with a factor of 8 for the tensor cores'
+truncation."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import denoiser as odn
+from test_gpu_kernels import _check_f16, _f, _rand
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2609_29505_gb300 import binding, build
+    build.build()
+    binding.lib()
+    return binding
+
+
+# widths 128 (smallest, one column tile of 8, ragged), 160, 192, 224, 256
+SHAPES = [(129, 8, 8), (300, 520, 688), (2000, 1272, 328), (2048, 3456, 72), (2040, 3840, 136), (2048, 4600, 136),
+          (4000, 4096, 264), (4128, 4088, 512), (4128, 1016, 4096)]
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
+@pytest.mark.parametrize("epi", ["f16", "f32", "gelu", "delta", "gate"])
+def test_pair_plain_and_residual(B, M, N, K, epi):
+    rng = np.random.default_rng(M + N + K)
+    A, W = _rand(rng, (M, K)).cuda(), _rand(rng, (N, K), 1 / math.sqrt(K)).cuda()
+    rows = np.unique(np.r_[0, 127, 128, M - 1, rng.choice(M, min(M, 200), replace=False)])
+    want = odn.linear(_f(A[rows]), _f(W))
+    tol = 8 * 2.0 ** -23 * math.sqrt(K) + 1e-6  # of results of unit scale
+    if epi in ("delta", "gate"):
+        h = torch.from_numpy(rng.standard_normal((M, N)).astype(np.float32)).cuda()
+        h0, cache = _f(h[rows]), torch.zeros(M, N, dtype=torch.float16, device="cuda")
+        e = B.sgd_epilogue_args(kind=B.EPI_DELTA, h=h.data_ptr(), ldh=N, cache=cache.data_ptr(), ld_cache=N)
+        if epi == "gate":  # samples of 100 rows: one or two per 32-row warp
+            g = torch.from_numpy(rng.standard_normal((-(-M // 100), N)).astype(np.float32)).cuda()
+            e.gate, e.ld_gate, e.rows_per_batch = g.data_ptr(), N, 100
+            want = want * _f(g)[rows // 100]
+        B.sgd_kernel_gemm(A, W, M, N, K, e)
+        np.testing.assert_allclose(_f(h[rows]), h0 + want, rtol=2e-6, atol=6 * tol)
+        _check_f16(cache[rows], want, extra_abs=6 * tol)
+    else:
+        out = torch.full((M, N), 7.0, dtype=torch.float32 if epi == "f32" else torch.float16, device="cuda")
+        kind = {"f16": B.EPI_F16, "f32": B.EPI_F32, "gelu": B.EPI_GELU}[epi]
+        B.sgd_kernel_gemm(A, W, M, N, K, B.sgd_epilogue_args(kind=kind, out=out.data_ptr(), ldo=N))
+        if epi == "f32":
+            np.testing.assert_allclose(_f(out[rows]), want, rtol=2e-6, atol=6 * tol)
+        else:
+            # the activations' fast exponential: 2^-21 relative
+            _check_f16(out[rows], odn.gelu_tanh(want) if epi == "gelu" else want, extra_abs=6 * tol + 2e-6)
+    torch.cuda.synchronize()
+    assert B.sgd_kernel_status() == 0
+
+
+@pytest.mark.parametrize("M,N,K", [(510, 8, 32), (2048, 1376, 136), (4096, 4600, 72)])
+@pytest.mark.parametrize("act", [0, 1])
+def test_pair_gated(B, M, N, K, act):
+    rng = np.random.default_rng(M + N + K + act)
+    A, W = _rand(rng, (M, K)).cuda(), _rand(rng, (2 * N, K), 1 / math.sqrt(K)).cuda()
+    out = torch.full((M, N), 7.0, dtype=torch.float16, device="cuda")
+    B.sgd_kernel_gemm(A, W, M, N, K, B.sgd_epilogue_args(kind=B.EPI_GATED, out=out.data_ptr(), ldo=N, act=act))
+    rows = np.unique(np.r_[0, 127, 128, M - 1, rng.choice(M, 200, replace=False)])
+    u = odn.linear(_f(A[rows]), _f(W))
+    want = u[:, :N] * odn.gelu_erf(u[:, N:]) if act else odn.silu(u[:, :N]) * u[:, N:]
+    _check_f16(out[rows], want, extra_abs=2e-5 * float(np.abs(want).max()))
+    assert B.sgd_kernel_status() == 0
+
+
+@pytest.mark.parametrize("dh", [64, 128])
+@pytest.mark.parametrize("M,heads,K", [(129, 1, 16), (437, 5, 72), (2048, 8, 264)])
+def test_pair_rope(B, M, heads, K, dh):
+    rng = np.random.default_rng(M + heads + K + dh)
+    N, tokens, half = 3 * heads * dh, 50, dh // 2
+    A, W = _rand(rng, (M, K)).cuda(), _rand(rng, (N, K), 1 / math.sqrt(K)).cuda()
+    ang = rng.standard_normal((tokens, half)).astype(np.float32)
+    cos, sin = (torch.from_numpy(f(ang)).cuda() for f in (np.cos, np.sin))
+    out = torch.full((M, N), 7.0, dtype=torch.float16, device="cuda")
+    e = B.sgd_epilogue_args(kind=B.EPI_ROPE, out=out.data_ptr(), ldo=N, rope_cos=cos.data_ptr(),
+                            rope_sin=sin.data_ptr(), rope_tokens=tokens, d_head=dh, rope_cols=2 * heads * dh)
+    B.sgd_kernel_gemm(A, W, M, N, K, e)
+    u = odn.linear(_f(A), _f(W)).reshape(M, 3 * heads, dh)
+    c, s = _f(cos)[np.arange(M) % tokens][:, None], _f(sin)[np.arange(M) % tokens][:, None]
+    r = u[:, :2 * heads]
+    rot = np.concatenate([r[..., :half] * c - r[..., half:] * s, r[..., half:] * c + r[..., :half] * s], -1)
+    want = np.concatenate([rot, u[:, 2 * heads:]], 1).reshape(M, N)
+    _check_f16(out, want, extra_abs=2e-5)
+    assert B.sgd_kernel_status() == 0
