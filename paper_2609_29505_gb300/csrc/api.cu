@@ -190,6 +190,7 @@ struct sgd_ctx {
   float* rope_cos = nullptr;
   float* rope_sin = nullptr;
   IoSlot* slot = nullptr;
+  TimeEmb temb;          // the step's time embeddings: of width d (stems), then t_freq (AdaLN)
   std::vector<f16*> cache;
   std::vector<f16*> ctxkv;
   std::vector<f16*> skipcat;
@@ -573,6 +574,7 @@ int build_program(sgd_ctx* c, const std::vector<uint8_t>& active, const std::vec
     p.pos = B16(c->w.pos_emb);
     p.class_emb = B16(c->w.class_emb);
     p.embed = B16(c->w.embed);
+    p.time = c->temb.out;
     p.vocab = d.vocab;
     p.n_classes = d.n_classes;
     Op op;
@@ -589,7 +591,8 @@ int build_program(sgd_ctx* c, const std::vector<uint8_t>& active, const std::vec
     GemvParams g{};
     g.out = c->t_hidden;
     g.ldo = D;
-    g.x_sinusoid = 1;
+    g.x = c->temb.out + c->temb.dim0;
+    g.ldx = 0;
     g.slot = c->slot;
     g.W = B16(c->w.w_t1);
     g.N = D;
@@ -927,6 +930,22 @@ int ensure_alloc(sgd_ctx* c) {
   if ((rc = c->alloc(&c->act, M * F, &c->ws_bytes))) return rc;
   if ((rc = c->alloc(&c->slot, 1, &c->ws_bytes))) return rc;
   CUDA_TRY(cudaMemset(c->slot, 0, sizeof(IoSlot)));
+  {
+    const int d0 = (d.stem == SGD_STEM_TIME_ADD || d.stem == SGD_STEM_PATCH_TOKENS) ? d.d : 0;
+    const int d1 = d.block == SGD_BLOCK_ADALN ? d.t_freq : 0;
+    c->temb.dim0 = d0;
+    c->temb.n = d0 + d1;
+    if (c->temb.n > 0) {
+      std::vector<double> w;
+      for (int dim : {d0, d1})
+        for (int i = 0; i < dim / 2; ++i) w.push_back(std::exp(-std::log(10000.0) * i / (dim / 2)));
+      double* wd = nullptr;
+      if ((rc = c->alloc(&c->temb.out, c->temb.n, &c->ws_bytes)) || (rc = c->alloc(&wd, w.size(), &c->ws_bytes)))
+        return rc;
+      CUDA_TRY(cudaMemcpy(wd, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice));
+      c->temb.w = wd;
+    }
+  }
   if (c->fold) {
     if ((rc = c->alloc(&c->h16, M * D, &c->ws_bytes))) return rc;
     if ((rc = c->alloc(&c->rstat, 2 * static_cast<size_t>(kStatSlots) * M, &c->ws_bytes))) return rc;
@@ -1130,7 +1149,7 @@ int prepare_step(sgd_ctx* c, const void* in, void* out, float t, const sgd_cond*
   v.ctx = cond ? cond->ctx : nullptr;
   v.t = t;
   v.step = step;
-  CUDA_TRY(io_set_launch(c->slot, v, s));
+  CUDA_TRY(io_set_launch(c->slot, v, c->temb, s));
   if (step == 1 && c->d.block == SGD_BLOCK_XATTN) {
     const int64_t n = static_cast<int64_t>(c->d.batch) * c->d.ctx_len * c->d.d_ctx;
     CUDA_TRY(convert_bf16_f16_launch(B16(cond->ctx), c->ctx16, n, 0, s));

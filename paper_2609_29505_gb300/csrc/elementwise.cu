@@ -4,8 +4,7 @@
 //                  (16-byte vectors: 8 fp32 of h, 8 fp16 of each cached update).
 //   frozen_rows  — the same for models whose pre-norms are folded into the GEMMs, also
 //                  writing fp16(h) and the partial row sums the next GEMM normalises with.
-//   norm         — pre-norm of an active branch where it cannot be folded (the AdaLN
-//                  modulate of DiT-style blocks), fp32 residual in, fp16 GEMM operand out.
+//   norm         — pre-norm of an active branch, fp32 residual in, fp16 GEMM operand out.
 //   stem, gemv, head_small, copy_out, pack_f16 — the always-on parts around the
 //                  scheduled units (input stage, conditioning, output head, U-ViT skip
 //                  operands), Sec. 4.2: conditioning and skip features stay current.
@@ -18,9 +17,6 @@
 namespace sgd {
 
 namespace {
-
-constexpr int kNormThreads = 128;
-constexpr int kNormMaxVec = 8;  // float4 per thread: d <= 4096
 
 __device__ __forceinline__ float block_sum(float v, float* red) {
 #pragma unroll
@@ -44,7 +40,7 @@ __device__ __forceinline__ void load_bf16x4(const bf16* p, float* f) {
 
 // y = ((x - mean) * rstd) * g + b, then * (1 + scale) + shift (AdaLN), for the 4 columns
 // 4 i .. 4 i + 3 of a row; sc / sh point at the row's sample's modulation (or are null).
-template <class P>  // NormParams or HeadParams (g, b: bf16 [d] or null)
+template <class P>  // HeadParams (g, b: bf16 [d] or null)
 __device__ __forceinline__ float4 norm_affine4(const P& p, int i, float4 v, float mean, float rstd,
                                                const float* sc, const float* sh) {
   float y[4] = {(v.x - mean) * rstd, (v.y - mean) * rstd, (v.z - mean) * rstd, (v.w - mean) * rstd};
@@ -71,112 +67,193 @@ __device__ __forceinline__ float4 norm_affine4(const P& p, int i, float4 v, floa
   return make_float4(y[0], y[1], y[2], y[3]);
 }
 
-// The same with the AdaLN modulation read as scalars (any alignment of shift / scale).
-__device__ __forceinline__ float4 norm_affine_s(const NormParams& p, int i, float4 v, float mean, float rstd,
-                                                const float* sc, const float* sh) {
-  float y[4] = {(v.x - mean) * rstd, (v.y - mean) * rstd, (v.z - mean) * rstd, (v.w - mean) * rstd};
-  if (p.g) {
-    float g[4];
-    load_bf16x4(p.g + 4 * i, g);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) y[k] *= g[k];
-  }
-  if (p.b) {
-    float b[4];
-    load_bf16x4(p.b + 4 * i, b);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) y[k] += b[k];
-  }
-  if (sc) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) y[k] = y[k] * (1.f + sc[4 * i + k]) + sh[4 * i + k];
-  }
-  return make_float4(y[0], y[1], y[2], y[3]);
-}
-
 __device__ __forceinline__ void store_f16x4(f16* p, float4 v) { *reinterpret_cast<uint2*>(p) = pack_f16x4(v); }
 
-__global__ void __launch_bounds__(kNormThreads) norm_kernel(const NormParams p) {
-  __shared__ float red[kNormThreads / 32];
-  pdl_wait_and_trigger();
-  const int row = blockIdx.x;
-  const int nv = p.d >> 2;
-  const float4* hr = reinterpret_cast<const float4*>(p.h + static_cast<int64_t>(row) * p.d);
-  float4 v[kNormMaxVec];
-  float sum = 0.f;
-#pragma unroll
-  for (int j = 0; j < kNormMaxVec; ++j) {
-    const int i = threadIdx.x + j * kNormThreads;
-    if (i < nv) {
-      v[j] = hr[i];
-      sum += (v[j].x + v[j].y) + (v[j].z + v[j].w);
+// The affine part's parameters for the 4 columns 4 i .. of a row, read ahead of the row's
+// statistics.  MODE: kGain bf16 gain and shift (either may be absent), no modulation; kMod an
+// AdaLN modulation in 16-byte vectors, no gain or shift; kAny everything, the modulation as
+// scalars at any alignment.
+enum { kGain = 0, kMod = 1, kAny = 2 };
+template <int MODE>
+struct Affine4 {
+  uint2 g, b;
+  float4 sc, sh;
+};
+template <>
+struct Affine4<kGain> {
+  uint2 g, b;
+};
+template <>
+struct Affine4<kMod> {
+  float4 sc, sh;
+};
+template <int MODE>
+__device__ __forceinline__ Affine4<MODE> load_affine4(const NormParams& p, int i, const float* sc, const float* sh) {
+  Affine4<MODE> a;
+  if constexpr (MODE != kMod) {
+    if (p.g) a.g = __ldg(reinterpret_cast<const uint2*>(p.g + 4 * i));
+    if (p.b) a.b = __ldg(reinterpret_cast<const uint2*>(p.b + 4 * i));
+  }
+  if constexpr (MODE == kMod) {
+    a.sc = __ldg(reinterpret_cast<const float4*>(sc + 4 * i));
+    a.sh = __ldg(reinterpret_cast<const float4*>(sh + 4 * i));
+  }
+  if constexpr (MODE == kAny) {
+    if (sc) {
+      a.sc = make_float4(sc[4 * i], sc[4 * i + 1], sc[4 * i + 2], sc[4 * i + 3]);
+      a.sh = make_float4(sh[4 * i], sh[4 * i + 1], sh[4 * i + 2], sh[4 * i + 3]);
     }
   }
-  float mean = 0.f, rstd;
-  if (p.kind == SGD_NORM_RMS) {
-    float sq = 0.f;
-#pragma unroll
-    for (int j = 0; j < kNormMaxVec; ++j) {
-      const int i = threadIdx.x + j * kNormThreads;
-      if (i < nv) sq += (v[j].x * v[j].x + v[j].y * v[j].y) + (v[j].z * v[j].z + v[j].w * v[j].w);
+  return a;
+}
+__device__ __forceinline__ float4 bf16x4(uint2 u) {
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 c = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, c.x, c.y);
+}
+template <int MODE>
+__device__ __forceinline__ float4 norm_apply4(const NormParams& p, const Affine4<MODE>& a, bool mod, float4 v,
+                                              float mean, float rstd) {
+  float4 y = make_float4((v.x - mean) * rstd, (v.y - mean) * rstd, (v.z - mean) * rstd, (v.w - mean) * rstd);
+  if constexpr (MODE != kMod) {
+    if (p.g) {
+      const float4 g = bf16x4(a.g);
+      y.x *= g.x; y.y *= g.y; y.z *= g.z; y.w *= g.w;
     }
-    sq = block_sum(sq, red);
-    rstd = rsqrtf(sq / p.d + p.eps);
-  } else {
-    mean = block_sum(sum, red) / p.d;
+    if (p.b) {
+      const float4 b = bf16x4(a.b);
+      y.x += b.x; y.y += b.y; y.z += b.z; y.w += b.w;
+    }
+  }
+  if constexpr (MODE != kGain) {
+    if (mod) {
+      y.x = y.x * (1.f + a.sc.x) + a.sh.x;
+      y.y = y.y * (1.f + a.sc.y) + a.sh.y;
+      y.z = y.z * (1.f + a.sc.z) + a.sh.z;
+      y.w = y.w * (1.f + a.sc.w) + a.sh.w;
+    }
+  }
+  return y;
+}
+
+// Rows wider than 2048 (LLaDA's 4096): 256 threads per row, kWideVec float4 each, and a grid of
+// a few blocks per SM that walk over the rows with the next row's loads in flight while the
+// current one is reduced and stored.  One block per row left the loads of a block's only row
+// exposed and a second, two-thirds full wave (4096 x 4096: 23.6 us against 19.2; bound by HBM).
+// Rows that fit in one wave of blocks get a block of 128 threads each (kPipe false).
+constexpr int wide_threads(bool pipe) { return pipe ? 256 : 128; }  // d <= 4096: 4 or 8 float4 per thread
+constexpr int wide_blocks(bool pipe) { return pipe ? 3 : 8; }  // per SM
+template <int MODE, bool kPipe>
+__global__ void __launch_bounds__(wide_threads(kPipe), wide_blocks(kPipe)) norm_wide_kernel(const NormParams p) {
+  constexpr int kThreads = wide_threads(kPipe), kVec = 1024 / kThreads;
+  __shared__ float red[2][kThreads / 32];
+  pdl_wait_and_trigger();
+  const int nv = p.d >> 2, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float inv_d = 1.f / p.d;
+  int flip = 0;
+  auto block_total = [&](float v) {  // one barrier per reduction: the buffers alternate
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[flip][warp] = v;
+    __syncthreads();
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < kThreads / 32; ++i) s += red[flip][i];
+    flip ^= 1;
+    return s;
+  };
+  float4 next[kVec];  // kPipe: the next row
+  auto fetch = [&](int row) {
+    const float4* hr = reinterpret_cast<const float4*>(p.h + static_cast<int64_t>(row) * p.d);
+#pragma unroll
+    for (int j = 0; j < kVec; ++j) {
+      const int i = threadIdx.x + j * kThreads;
+      next[j] = i < nv ? hr[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  if (static_cast<int>(blockIdx.x) < p.rows) fetch(blockIdx.x);
+  for (int row = blockIdx.x; row < p.rows; row += gridDim.x) {
+    float4 v[kVec];
+#pragma unroll
+    for (int j = 0; j < kVec; ++j) v[j] = next[j];
+    const int64_t smp = p.scale ? row / p.rows_per_batch : 0;
+    const float* sh = p.shift ? p.shift + smp * p.ld_mod : nullptr;
+    const float* sc = p.scale ? p.scale + smp * p.ld_mod : nullptr;
+    Affine4<MODE> af[kPipe ? kVec : 1];
+    if (kPipe) {
+#pragma unroll
+      for (int j = 0; j < kVec; ++j) {
+        const int i = threadIdx.x + j * kThreads;
+        if (i < nv) af[kPipe ? j : 0] = load_affine4<MODE>(p, i, sc, sh);
+      }
+    }
+    if (kPipe && row + gridDim.x < p.rows) fetch(row + gridDim.x);
+    float mean = 0.f, sum = 0.f;
+    if (p.kind != SGD_NORM_RMS) {
+#pragma unroll
+      for (int j = 0; j < kVec; ++j) sum += (v[j].x + v[j].y) + (v[j].z + v[j].w);
+      mean = block_total(sum) * inv_d;
+    }
     float sq = 0.f;
 #pragma unroll
-    for (int j = 0; j < kNormMaxVec; ++j) {
-      const int i = threadIdx.x + j * kNormThreads;
-      if (i < nv) {
+    for (int j = 0; j < kVec; ++j) {
+      if (static_cast<int>(threadIdx.x) + j * kThreads < nv) {
         const float a = v[j].x - mean, b = v[j].y - mean, c = v[j].z - mean, d = v[j].w - mean;
         sq += (a * a + b * b) + (c * c + d * d);
       }
     }
-    sq = block_sum(sq, red);
-    rstd = rsqrtf(sq / p.d + p.eps);
-  }
-  const float* sh = p.shift ? p.shift + static_cast<int64_t>(row / p.rows_per_batch) * p.ld_mod : nullptr;
-  const float* sc = p.scale ? p.scale + static_cast<int64_t>(row / p.rows_per_batch) * p.ld_mod : nullptr;
-  f16* orow = p.out + static_cast<int64_t>(row) * p.d;
-  // (the fp16 stores cannot alias the fp32 / bf16 parameter loads, so the compiler issues
-  // those loads ahead of the stores; transforming every vector before the first store
-  // measured slower)
+    const float rstd = rsqrtf(block_total(sq) * inv_d + p.eps);
+    f16* orow = p.out + static_cast<int64_t>(row) * p.d;
 #pragma unroll
-  for (int j = 0; j < kNormMaxVec; ++j) {
-    const int i = threadIdx.x + j * kNormThreads;
-    if (i < nv) store_f16x4(orow + 4 * i, norm_affine_s(p, i, v[j], mean, rstd, sc, sh));
+    for (int j = 0; j < kVec; ++j) {
+      const int i = threadIdx.x + j * kThreads;
+      if (i < nv) {
+        const Affine4<MODE> a = kPipe ? af[kPipe ? j : 0] : load_affine4<MODE>(p, i, sc, sh);
+        store_f16x4(orow + 4 * i, norm_apply4<MODE>(p, a, sc != nullptr, v[j], mean, rstd));
+      }
+    }
   }
 }
 
-// Same normalisation with one warp per row (d <= 2048: at most 16 float4 per lane), one
-// row per warp of the block: no block-wide reductions, and for the 1-2 k-wide rows of the mid-size
-// models a 128-thread block per row would leave each thread two vectors of work.
-constexpr int kNormWarpMaxVec = 16;
-__global__ void __launch_bounds__(256) norm_warp_kernel(const NormParams p) {
+// One warp per row (d <= 2048, NV float4 per lane): no block-wide reductions.  The row's
+// modulation is read with the row, ahead of its statistics (reading them after, the
+// modulation as scalars, took 6.2 us for 2048 x 1152 against the launch's ~2.5 us of traffic).
+template <int NV, int MODE>
+__global__ void __launch_bounds__(128, MODE != kGain ? 4 : (NV <= 8 ? 8 : 5)) norm_warp_kernel(const NormParams p) {
   pdl_wait_and_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * (blockDim.x >> 5) + warp;
   if (row >= p.rows) return;
   const int nv = p.d >> 2;
   const float4* hr = reinterpret_cast<const float4*>(p.h + static_cast<int64_t>(row) * p.d);
-  float4 v[kNormWarpMaxVec];
-  float sum = 0.f, sq = 0.f;
+  const int64_t smp = p.scale ? row / p.rows_per_batch : 0;
+  const float* sh = p.shift ? p.shift + smp * p.ld_mod : nullptr;
+  const float* sc = p.scale ? p.scale + smp * p.ld_mod : nullptr;
+  float4 v[NV];
 #pragma unroll
-  for (int j = 0; j < kNormWarpMaxVec; ++j) {
+  for (int j = 0; j < NV; ++j) {
     const int i = lane + 32 * j;
-    if (i < nv) {
-      v[j] = hr[i];
-      sum += (v[j].x + v[j].y) + (v[j].z + v[j].w);
+    v[j] = i < nv ? hr[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // (a gain is the same for all rows, in L1 after the first; registers are better spent on rows)
+  constexpr bool kAhead = NV <= 10 && MODE == kMod;
+  Affine4<MODE> af[kAhead ? NV : 1];
+  if (kAhead) {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int i = lane + 32 * j;
+      if (i < nv) af[kAhead ? j : 0] = load_affine4<MODE>(p, i, sc, sh);
     }
   }
+  float sum = 0.f, sq = 0.f;
+#pragma unroll
+  for (int j = 0; j < NV; ++j) sum += (v[j].x + v[j].y) + (v[j].z + v[j].w);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   const float mean = p.kind == SGD_NORM_RMS ? 0.f : sum / p.d;
 #pragma unroll
-  for (int j = 0; j < kNormWarpMaxVec; ++j) {
-    const int i = lane + 32 * j;
-    if (i < nv) {
+  for (int j = 0; j < NV; ++j) {
+    if (lane + 32 * j < nv) {
       const float a = v[j].x - mean, b = v[j].y - mean, c = v[j].z - mean, d = v[j].w - mean;
       sq += (a * a + b * b) + (c * c + d * d);
     }
@@ -184,13 +261,14 @@ __global__ void __launch_bounds__(256) norm_warp_kernel(const NormParams p) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
   const float rstd = rsqrtf(sq / p.d + p.eps);
-  const float* sh = p.shift ? p.shift + static_cast<int64_t>(row / p.rows_per_batch) * p.ld_mod : nullptr;
-  const float* sc = p.scale ? p.scale + static_cast<int64_t>(row / p.rows_per_batch) * p.ld_mod : nullptr;
   f16* orow = p.out + static_cast<int64_t>(row) * p.d;
 #pragma unroll
-  for (int j = 0; j < kNormWarpMaxVec; ++j) {
+  for (int j = 0; j < NV; ++j) {
     const int i = lane + 32 * j;
-    if (i < nv) store_f16x4(orow + 4 * i, norm_affine_s(p, i, v[j], mean, rstd, sc, sh));
+    if (i < nv) {
+      const Affine4<MODE> a = kAhead ? af[kAhead ? j : 0] : load_affine4<MODE>(p, i, sc, sh);
+      store_f16x4(orow + 4 * i, norm_apply4<MODE>(p, a, sc != nullptr, v[j], mean, rstd));
+    }
   }
 }
 
@@ -338,17 +416,27 @@ __global__ void __launch_bounds__(256) frozen_rows_kernel(const __grid_constant_
   }
 }
 
-__global__ void io_set_kernel(IoSlot* slot, const IoSlot v) { *slot = v; }
-
-// sinusoid(t, dim)[c] = cos(t w_i) for c < half, sin(t w_{c-half}) otherwise,
-// w_i = 10000^(-i / half), evaluated in double precision.
-__device__ __forceinline__ float sinusoid_at(double t, int dim, int c) {
+// Writes the step's I/O slot and its time embeddings sinusoid(t, dim)[c] = cos(t w_i) for c < half,
+// sin(t w_{c-half}) otherwise, w_i = 10000^(-i / half) (a table in double, made at creation).  The
+// cosine and sine are in double, at a few dozen results per clock for the whole GPU: formed here
+// once per step instead of by every block (or element) that reads them.
+__global__ void io_set_kernel(IoSlot* slot, const IoSlot v, const TimeEmb te) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *slot = v;
+  if (i >= te.n) return;
+  int dim = te.dim0, c = i;
+  const double* w = te.w;
+  if (c >= te.dim0) {
+    c -= te.dim0;
+    w += te.dim0 >> 1;
+    dim = te.n - te.dim0;
+  }
   const int half = dim >> 1;
-  const int i = c < half ? c : c - half;
-  const double w = exp(-9.210340371976184 * static_cast<double>(i) / half);  // ln(10000)
-  return static_cast<float>(c < half ? cos(t * w) : sin(t * w));
+  const double t = v.t;
+  te.out[i] = static_cast<float>(c < half ? cos(t * w[c]) : sin(t * w[c - half]));
 }
 
+// The stems of arbitrary widths: one thread per element.
 __global__ void stem_kernel(const StemParams p) {
   pdl_wait_and_trigger();
   const int64_t total = static_cast<int64_t>(p.batch) * p.n_tokens * p.d;
@@ -360,47 +448,118 @@ __global__ void stem_kernel(const StemParams p) {
   const int b = static_cast<int>(r / p.n_tokens);
   const IoSlot* s = p.slot;
   float v = 0.f;
-  switch (p.kind) {
-    case SGD_STEM_TIME_ADD:
-      v = reinterpret_cast<const float*>(s->state)[idx] + sinusoid_at(s->t, p.d, c);
-      break;
-    case SGD_STEM_IDENTITY:
-      v = reinterpret_cast<const float*>(s->state)[idx];
-      break;
-    case SGD_STEM_EMBED: {
-      const int id = min(max(reinterpret_cast<const int32_t*>(s->state)[r], 0), p.vocab - 1);
-      v = __bfloat162float(p.embed[static_cast<int64_t>(id) * p.d + c]);
-      break;
-    }
-    case SGD_STEM_PATCH:
-    case SGD_STEM_PATCH_TOKENS: {
-      const int np = n - p.n_prefix;
-      if (np < 0) {
-        const int cls = min(max(s->class_ids[b], 0), p.n_classes - 1);
-        v = (n == 0) ? sinusoid_at(s->t, p.d, c)
-                     : __bfloat162float(p.class_emb[static_cast<int64_t>(cls) * p.d + c]);
-      } else {
-        const float* z = reinterpret_cast<const float*>(s->state) +
-                         (static_cast<int64_t>(b) * (p.n_tokens - p.n_prefix) + np) * p.d_in;
-        const bf16* w = p.w_stem + static_cast<int64_t>(c) * p.d_in;
-        float acc = 0.f;
-        for (int k = 0; k < p.d_in; ++k) acc = fmaf(z[k], __bfloat162float(w[k]), acc);
-        v = acc;
-      }
-      v += __bfloat162float(p.pos[static_cast<int64_t>(n) * p.d + c]);
-      break;
-    }
-    default:
-      break;
+  const int np = n - p.n_prefix;
+  if (np < 0) {
+    const int cls = min(max(s->class_ids[b], 0), p.n_classes - 1);
+    v = (n == 0) ? p.time[c]
+                 : __bfloat162float(p.class_emb[static_cast<int64_t>(cls) * p.d + c]);
+  } else {
+    const float* z = reinterpret_cast<const float*>(s->state) +
+                     (static_cast<int64_t>(b) * (p.n_tokens - p.n_prefix) + np) * p.d_in;
+    const bf16* w = p.w_stem + static_cast<int64_t>(c) * p.d_in;
+    float acc = 0.f;
+    for (int k = 0; k < p.d_in; ++k) acc = fmaf(z[k], __bfloat162float(w[k]), acc);
+    v = acc;
   }
+  v += __bfloat162float(p.pos[static_cast<int64_t>(n) * p.d + c]);
   p.h[idx] = v;
 }
 
-// The patch stems with one thread per (token row, 4 channels): the row's d_in patch values
-// and the 4 channels' weight rows are read as 16-byte vectors (d_in % 8 == 0, d % 4 == 0),
-// each channel's dot product is summed in k order exactly as in stem_kernel, and the 4
-// results go out as one float4.
-__global__ void stem_patch_kernel(const StemParams p) {
+// The stems without a projection (d % 8 == 0), bound by writing h: thread (x, y) handles 8
+// columns of every gridDim.y-th row in 16-byte vectors (4096 x 4096 embedding rows: 72 us with
+// one element per thread).
+__global__ void __launch_bounds__(128) stem_rows_kernel(const StemParams p) {
+  pdl_wait_and_trigger();
+  const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * 8;
+  if (c0 >= p.d) return;
+  const IoSlot* s = p.slot;
+  const int rows = p.batch * p.n_tokens;
+  float4 ta = make_float4(0.f, 0.f, 0.f, 0.f), tb = ta;
+  if (p.kind == SGD_STEM_TIME_ADD) {
+    ta = *reinterpret_cast<const float4*>(p.time + c0);
+    tb = *reinterpret_cast<const float4*>(p.time + c0 + 4);
+  }
+  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+    const int64_t at = static_cast<int64_t>(r) * p.d + c0;
+    float4 a, b;
+    if (p.kind == SGD_STEM_EMBED) {
+      const int id = min(max(reinterpret_cast<const int32_t*>(s->state)[r], 0), p.vocab - 1);
+      const uint4 u = __ldg(reinterpret_cast<const uint4*>(p.embed + static_cast<int64_t>(id) * p.d + c0));
+      a = bf16x4(make_uint2(u.x, u.y));
+      b = bf16x4(make_uint2(u.z, u.w));
+    } else {
+      const float4* z = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(s->state) + at);
+      a = z[0];
+      b = z[1];
+      if (p.kind == SGD_STEM_TIME_ADD) {
+        a.x += ta.x; a.y += ta.y; a.z += ta.z; a.w += ta.w;
+        b.x += tb.x; b.y += tb.y; b.z += tb.z; b.w += tb.w;
+      }
+    }
+    float4* h = reinterpret_cast<float4*>(p.h + at);
+    h[0] = a;
+    h[1] = b;
+  }
+}
+
+// The patch stems (d_in % 8 == 0, d % 4 == 0), bound by writing h: a thread owns 4 channels, with
+// their DIN-wide weight rows in registers, and a block walks over kPatchRows token rows whose
+// patches it has put in shared memory (read by every thread alike).  One thread per (row, 4
+// channels) read its 4 weight rows again for every row, 32 different lines per load: 22 us for
+// 2048 x 1152.  Each channel's dot product is summed in k order as in stem_kernel.
+constexpr int kPatchRows = 16;
+template <int DIN>
+__global__ void __launch_bounds__(128) stem_patch_kernel(const StemParams p) {
+  __shared__ float4 zs[kPatchRows][DIN / 4];
+  pdl_wait_and_trigger();
+  const IoSlot* s = p.slot;
+  const int rows = p.batch * p.n_tokens, r0 = blockIdx.y * kPatchRows, nr = min(kPatchRows, rows - r0);
+  const int n_in = p.n_tokens - p.n_prefix;
+  for (int i = threadIdx.x; i < nr * (DIN / 4); i += blockDim.x) {
+    const int k = i / (DIN / 4), r = r0 + k;
+    const int n = r % p.n_tokens - p.n_prefix, b = r / p.n_tokens;
+    if (n >= 0)
+      zs[k][i % (DIN / 4)] = reinterpret_cast<const float4*>(s->state)[(static_cast<int64_t>(b) * n_in + n) * (DIN / 4) + i % (DIN / 4)];
+  }
+  const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  const bool active = c0 < p.d;
+  float w[4][DIN];
+  if (active) {
+    const uint4* wp = reinterpret_cast<const uint4*>(p.w_stem + static_cast<int64_t>(c0) * DIN);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int k8 = 0; k8 < DIN / 8; ++k8) unpack_bf16x8(__ldg(wp + q * (DIN / 8) + k8), &w[q][8 * k8]);
+  }
+  __syncthreads();
+  if (!active) return;
+#pragma unroll 1
+  for (int k = 0; k < nr; ++k) {
+    const int r = r0 + k, n = r % p.n_tokens, b = r / p.n_tokens;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n < p.n_prefix) {
+      const int cls = min(max(s->class_ids[b], 0), p.n_classes - 1);
+      v = n == 0 ? *reinterpret_cast<const float4*>(p.time + c0)
+                 : bf16x4(*reinterpret_cast<const uint2*>(p.class_emb + static_cast<int64_t>(cls) * p.d + c0));
+    } else {
+#pragma unroll
+      for (int i = 0; i < DIN / 4; ++i) {
+        const float4 z = zs[k][i];
+        v.x = fmaf(z.w, w[0][4 * i + 3], fmaf(z.z, w[0][4 * i + 2], fmaf(z.y, w[0][4 * i + 1], fmaf(z.x, w[0][4 * i], v.x))));
+        v.y = fmaf(z.w, w[1][4 * i + 3], fmaf(z.z, w[1][4 * i + 2], fmaf(z.y, w[1][4 * i + 1], fmaf(z.x, w[1][4 * i], v.y))));
+        v.z = fmaf(z.w, w[2][4 * i + 3], fmaf(z.z, w[2][4 * i + 2], fmaf(z.y, w[2][4 * i + 1], fmaf(z.x, w[2][4 * i], v.z))));
+        v.w = fmaf(z.w, w[3][4 * i + 3], fmaf(z.z, w[3][4 * i + 2], fmaf(z.y, w[3][4 * i + 1], fmaf(z.x, w[3][4 * i], v.w))));
+      }
+    }
+    const float4 ps = bf16x4(__ldg(reinterpret_cast<const uint2*>(p.pos + static_cast<int64_t>(n) * p.d + c0)));
+    *reinterpret_cast<float4*>(p.h + static_cast<int64_t>(r) * p.d + c0) =
+        make_float4(v.x + ps.x, v.y + ps.y, v.z + ps.z, v.w + ps.w);
+  }
+}
+
+// Patch widths without an instantiation above (d_in % 8 == 0): one thread per (token row, 4
+// channels), the row's patch and the 4 channels' weight rows read as 16-byte vectors.
+__global__ void stem_patch_any_kernel(const StemParams p) {
   pdl_wait_and_trigger();
   const int d4 = p.d >> 2;
   const int64_t total = static_cast<int64_t>(p.batch) * p.n_tokens * d4;
@@ -417,7 +576,7 @@ __global__ void stem_patch_kernel(const StemParams p) {
     const int cls = min(max(s->class_ids[b], 0), p.n_classes - 1);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      v[q] = (n == 0) ? sinusoid_at(s->t, p.d, c0 + q)
+      v[q] = (n == 0) ? p.time[c0 + q]
                       : __bfloat162float(p.class_emb[static_cast<int64_t>(cls) * p.d + c0 + q]);
   } else {
     const float4* z = reinterpret_cast<const float4*>(
@@ -452,7 +611,21 @@ __global__ void stem_patch_kernel(const StemParams p) {
 // x is staged as two planes (k % 8 < 4, k % 8 >= 4) so that the lanes' 16-byte x loads are
 // consecutive (no bank conflicts).  With 8 rows the warp's 4 x 8 partial sums are reduced by
 // a transpose reduction (31 shuffles, lane l ends with value l) instead of 32 butterflies.
-constexpr int kGemvCols = 4;
+//
+// The products are formed as pairs of even and odd k (fma.rn.f32x2, two fp32 fmas per
+// instruction, both halves added at the end): with one fma per instruction and 8 rows the fma
+// pipe came close to the weight stream's time.
+__device__ __forceinline__ uint64_t pack_f32x2(uint32_t lo, uint32_t hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+  return d;
+}
+__device__ __forceinline__ void fma_f32x2(uint64_t& d, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float sum_f32x2(uint64_t a) {
+  return __uint_as_float(static_cast<uint32_t>(a)) + __uint_as_float(static_cast<uint32_t>(a >> 32));
+}
 
 // v[0..31] of every lane -> lane l returns the warp's sum of value l
 __device__ __forceinline__ float transpose_reduce32(float* v, int lane) {
@@ -479,20 +652,16 @@ __device__ __forceinline__ void gemv_store(const GemvParams& p, float* out, int 
   if (p.out_silu) p.out_silu[static_cast<int64_t>(r) * p.ldo + j] = silu_f(v);
 }
 
-template <int RMAX>
+// COLS columns per warp: 32 / RMAX with several rows; for one row 4, or 1 where the columns are
+// too few to fill the SMs otherwise (the conditioning MLP: 1152 columns).
+template <int RMAX, int COLS>
 __global__ void __launch_bounds__(256) gemv_kernel(const GemvParams p) {
   extern __shared__ float xs[];  // [xrows][2 planes][K / 2]
   pdl_wait_and_trigger();
-  const int xrows = p.x_sinusoid ? 1 : (p.ldx == 0 ? 1 : p.rows);
+  const int xrows = p.ldx == 0 ? 1 : p.rows;
   const int K = p.K, half = K >> 1;
   // x[r][k] lives at r * K + (k & 4 ? half : 0) + (k >> 3) * 4 + (k & 3)
-  if (p.x_sinusoid) {
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-      float x = sinusoid_at(p.slot->t, K, k);
-      if (p.in_silu) x = silu_f(x);
-      xs[((k & 4) ? half : 0) + (k >> 3) * 4 + (k & 3)] = x;
-    }
-  } else {
+  {
     // float4 loads (K % 8 == 0, rows 16-byte aligned) in batches of 8 per thread, every load
     // of a batch issued before its first shared-memory store: x is a generic pointer that
     // the compiler cannot tell apart from xs, so a store in between would make each load
@@ -528,75 +697,64 @@ __global__ void __launch_bounds__(256) gemv_kernel(const GemvParams p) {
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kItemCols = 8 * kGemvCols;  // 8 warps
+  constexpr int kCols = COLS;
+  constexpr int kItemCols = 8 * kCols;  // 8 warps
   const int per_seg = (p.N + kItemCols - 1) / kItemCols;
   const int n_items = per_seg * (p.n_seg > 0 ? p.n_seg : 1);
   for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     const int seg = item / per_seg;
-    const int j0 = (item - seg * per_seg) * kItemCols + warp * kGemvCols;
+    const int j0 = (item - seg * per_seg) * kItemCols + warp * kCols;
     if (j0 >= p.N) continue;  // warp-uniform; no block-wide barrier follows
     const bf16* W = p.n_seg ? p.w_seg[seg] : p.W;
     float* out = p.n_seg ? p.out_seg[seg] : p.out;
-    float acc[kGemvCols * RMAX];
+    uint64_t acc2[kCols * RMAX];  // sums over even and odd k
 #pragma unroll
-    for (int i = 0; i < kGemvCols * RMAX; ++i) acc[i] = 0.f;
+    for (int i = 0; i < kCols * RMAX; ++i) acc2[i] = 0;
     // unrolled so that a warp's weight loads for several K steps are in flight together
 #pragma unroll 4
     for (int k = lane * 8; k < K; k += 256) {
-      float w[kGemvCols][8];
+      uint4 w[kCols];  // columns past N repeat the last one, whose sums are then not stored
 #pragma unroll
-      for (int c = 0; c < kGemvCols; ++c) {
-        if (j0 + c < p.N)
-          unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(W + static_cast<int64_t>(j0 + c) * K + k)), w[c]);
-        else
-#pragma unroll
-          for (int q = 0; q < 8; ++q) w[c][q] = 0.f;
-      }
+      for (int c = 0; c < kCols; ++c)
+        w[c] = __ldg(reinterpret_cast<const uint4*>(W + static_cast<int64_t>(min(j0 + c, p.N - 1)) * K + k));
       const int xo = (k >> 3) * 4;
+      uint64_t wf[kCols][4];
+#pragma unroll
+      for (int c = 0; c < kCols; ++c) {
+        const uint32_t u[4] = {w[c].x, w[c].y, w[c].z, w[c].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) wf[c][q] = pack_f32x2(u[q] << 16, u[q] & 0xffff0000u);
+      }
 #pragma unroll
       for (int r = 0; r < RMAX; ++r) {
         if (r < xrows) {
-          const float4 xa = *reinterpret_cast<const float4*>(xs + r * K + xo);
-          const float4 xb = *reinterpret_cast<const float4*>(xs + r * K + half + xo);
-          const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+          const ulonglong2 xa = *reinterpret_cast<const ulonglong2*>(xs + r * K + xo);
+          const ulonglong2 xb = *reinterpret_cast<const ulonglong2*>(xs + r * K + half + xo);
+          const uint64_t xv[4] = {xa.x, xa.y, xb.x, xb.y};
 #pragma unroll
-          for (int c = 0; c < kGemvCols; ++c)
+          for (int c = 0; c < kCols; ++c)
 #pragma unroll
-            for (int q = 0; q < 8; ++q) acc[c * RMAX + r] = fmaf(w[c][q], xv[q], acc[c * RMAX + r]);
+            for (int q = 0; q < 4; ++q) fma_f32x2(acc2[c * RMAX + r], wf[c][q], xv[q]);
         }
       }
     }
-    if constexpr (kGemvCols * RMAX == 32) {
+    float acc[kCols * RMAX];
+#pragma unroll
+    for (int i = 0; i < kCols * RMAX; ++i) acc[i] = sum_f32x2(acc2[i]);
+    if constexpr (kCols * RMAX == 32) {
       // lane l: column j0 + l / RMAX, row l % RMAX
       const float v = transpose_reduce32(acc, lane);
       const int c = lane / RMAX, r = lane % RMAX;
       if (r < p.rows && j0 + c < p.N) gemv_store(p, out, r, j0 + c, v);
-    } else {
+    } else {  // one row of x: the same products for every output row
+      static_assert(RMAX == 1 && kCols <= 4, "one row");
 #pragma unroll
-      for (int i = 0; i < kGemvCols * RMAX; ++i) {
-        if (i % RMAX < xrows) {
+      for (int c = 0; c < kCols; ++c)
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-        }
-      }
-      if (lane < kGemvCols && j0 + lane < p.N) {
-        const int j = j0 + lane;
-        // lane c stores column j0 + c; select chains keep acc in registers
-        float vals[RMAX];
+        for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
 #pragma unroll
-        for (int rr = 0; rr < RMAX; ++rr) {
-          float v = acc[rr];
-#pragma unroll
-          for (int c = 1; c < kGemvCols; ++c) v = (lane == c) ? acc[c * RMAX + rr] : v;
-          vals[rr] = v;
-        }
-        for (int r = 0; r < p.rows; ++r) {
-          float v = vals[0];
-#pragma unroll
-          for (int rr = 1; rr < RMAX; ++rr) v = (xrows > 1 && rr == r) ? vals[rr] : v;
-          gemv_store(p, out, r, j, v);
-        }
-      }
+      for (int c = 0; c < kCols; ++c)
+        if (lane < p.rows && j0 + c < p.N) gemv_store(p, out, lane, j0 + c, acc[c]);
     }
   }
 }
@@ -607,79 +765,77 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// One warp per row: the fp32 row is read once into registers (lane l holds columns 4 (l + 32 j)
-// .. + 3), its mean and rstd are reduced across the warp, the row is normalised (and AdaLN
-// modulated) in place, and then every output channel's dot product with it is formed from
-// the channel's bf16 weight row (read through the read-only cache: out_channels x K x 2
-// bytes, shared by all rows) and reduced across the warp; lane c keeps channel c (and
-// c + 32), and the row's outputs are stored together at the end.
-template <int MAXV>  // float4 per lane: K <= 128 MAXV
-__global__ void __launch_bounds__(256) head_small_kernel(const HeadParams p) {
+// A warp takes two rows: it normalises (and AdaLN modulates) them into its part of shared memory
+// and multiplies them by 16 output channels' bf16 weight rows at a time, whose loads serve both
+// rows (the weights come from L1: out_channels x K x 2 bytes per warp).  The 32 partial sums of a
+// lane are reduced over the warp by one transpose reduction, after which lane l holds channel
+// l / 2 of row l % 2.  One channel at a time, with its own reduction, was a chain of load and
+// shuffle latencies (29 us for 2048 x 1152 and 16 channels), and with the rows in registers the
+// unrolled code was as long as the work (26 us).
+__global__ void __launch_bounds__(128, 3) head_small_kernel(const HeadParams p) {
+  extern __shared__ float xh[];  // [warp][2][K]
   pdl_wait_and_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t r = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp;
+  const int64_t r0 = (static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp) * 2;
   const int64_t rows = static_cast<int64_t>(p.batch) * p.n_tokens;
-  if (r >= rows) return;
-  const int n = static_cast<int>(r % p.n_tokens), b = static_cast<int>(r / p.n_tokens);
-  if (n < p.n_prefix) return;
-  float* out = reinterpret_cast<float*>(p.slot->out) +
-               (static_cast<int64_t>(b) * (p.n_tokens - p.n_prefix) + (n - p.n_prefix)) *
-                   p.out_channels;
-  const float4* x = reinterpret_cast<const float4*>(p.h + r * p.ldx);
+  if (r0 >= rows) return;
   const int nv = p.K >> 2;
-  float4 v[MAXV];
-  float s1 = 0.f;
-#pragma unroll
-  for (int j = 0; j < MAXV; ++j) {
-    const int i = lane + 32 * j;
-    if (i < nv) {
-      v[j] = __ldg(x + i);
-      s1 += (v[j].x + v[j].y) + (v[j].z + v[j].w);
+  float4* x0 = reinterpret_cast<float4*>(xh + static_cast<size_t>(2 * warp) * p.K);
+#pragma unroll 1
+  for (int q = 0; q < 2; ++q) {
+    const int64_t r = min(r0 + q, rows - 1);  // past the last row: computed again, not stored
+    const int b = static_cast<int>(r / p.n_tokens);
+    const float4* x = reinterpret_cast<const float4*>(p.h + r * p.ldx);
+    float4* xs = x0 + q * nv;
+    float s1 = 0.f, sq = 0.f;
+#pragma unroll 4
+    for (int i = lane; i < nv; i += 32) {
+      const float4 v = __ldg(x + i);
+      xs[i] = v;
+      s1 += (v.x + v.y) + (v.z + v.w);
     }
-  }
-  const float mean = p.norm_kind != SGD_NORM_RMS ? warp_sum(s1) / p.K : 0.f;
-  float sq = 0.f;
-#pragma unroll
-  for (int j = 0; j < MAXV; ++j) {
-    const int i = lane + 32 * j;
-    if (i < nv) {
-      const float a0 = v[j].x - mean, a1 = v[j].y - mean, a2 = v[j].z - mean, a3 = v[j].w - mean;
+    const float mean = p.norm_kind != SGD_NORM_RMS ? warp_sum(s1) / p.K : 0.f;
+#pragma unroll 4
+    for (int i = lane; i < nv; i += 32) {
+      const float4 v = xs[i];
+      const float a0 = v.x - mean, a1 = v.y - mean, a2 = v.z - mean, a3 = v.w - mean;
       sq += (a0 * a0 + a1 * a1) + (a2 * a2 + a3 * a3);
     }
+    const float rstd = rsqrtf(warp_sum(sq) / p.K + p.eps);
+    const float* sh = p.shift ? p.shift + static_cast<int64_t>(b) * p.ld_mod : nullptr;
+    const float* sc = p.scale ? p.scale + static_cast<int64_t>(b) * p.ld_mod : nullptr;
+#pragma unroll 2
+    for (int i = lane; i < nv; i += 32) xs[i] = norm_affine4(p, i, xs[i], mean, rstd, sc, sh);
   }
-  const float rstd = rsqrtf(warp_sum(sq) / p.K + p.eps);
-  const float* sh = p.shift ? p.shift + static_cast<int64_t>(b) * p.ld_mod : nullptr;
-  const float* sc = p.scale ? p.scale + static_cast<int64_t>(b) * p.ld_mod : nullptr;
+  // this lane's output row and channel within a group (each lane reads back what it wrote)
+  const int64_t ro = r0 + (lane & 1);
+  const int n = static_cast<int>(ro % p.n_tokens), b = static_cast<int>(ro / p.n_tokens);
+  float* out = reinterpret_cast<float*>(p.slot->out) +
+               (static_cast<int64_t>(b) * (p.n_tokens - p.n_prefix) + (n - p.n_prefix)) * p.out_channels;
+  const bool store = ro < rows && n >= p.n_prefix;
+#pragma unroll 1
+  for (int c0 = 0; c0 < p.out_channels; c0 += 16) {
+    float acc[32];
 #pragma unroll
-  for (int j = 0; j < MAXV; ++j) {
-    const int i = lane + 32 * j;
-    if (i < nv) v[j] = norm_affine4(p, i, v[j], mean, rstd, sc, sh);
-  }
-  float res0 = 0.f, res1 = 0.f;
-  for (int c = 0; c < p.out_channels; ++c) {
-    const uint2* w = reinterpret_cast<const uint2*>(p.W + static_cast<int64_t>(c) * p.K);
-    float acc = 0.f;
+    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+#pragma unroll 2
+    for (int i = lane; i < nv; i += 32) {
+      uint2 w[16];  // channels past the last repeat it, not stored
 #pragma unroll
-    for (int j = 0; j < MAXV; ++j) {
-      const int i = lane + 32 * j;
-      if (i < nv) {
-        const uint2 u = __ldg(w + i);
-        const __nv_bfloat162* wb = reinterpret_cast<const __nv_bfloat162*>(&u);
-        const float2 w01 = __bfloat1622float2(wb[0]), w23 = __bfloat1622float2(wb[1]);
-        acc = fmaf(v[j].x, w01.x, acc);
-        acc = fmaf(v[j].y, w01.y, acc);
-        acc = fmaf(v[j].z, w23.x, acc);
-        acc = fmaf(v[j].w, w23.y, acc);
+      for (int c = 0; c < 16; ++c)
+        w[c] = __ldg(reinterpret_cast<const uint2*>(p.W + static_cast<int64_t>(min(c0 + c, p.out_channels - 1)) * p.K) + i);
+      const float4 u = x0[i], v = x0[nv + i];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const float4 wf = bf16x4(w[c]);
+        acc[2 * c] = fmaf(u.w, wf.w, fmaf(u.z, wf.z, fmaf(u.y, wf.y, fmaf(u.x, wf.x, acc[2 * c]))));
+        acc[2 * c + 1] = fmaf(v.w, wf.w, fmaf(v.z, wf.z, fmaf(v.y, wf.y, fmaf(v.x, wf.x, acc[2 * c + 1]))));
       }
     }
-    acc = warp_sum(acc);
-    if (c < 32)
-      res0 = lane == c ? acc : res0;
-    else
-      res1 = lane == c - 32 ? acc : res1;
+    const float res = transpose_reduce32(acc, lane);
+    const int c = c0 + (lane >> 1);
+    if (store && c < p.out_channels) out[c] = res;
   }
-  if (lane < p.out_channels) out[lane] = res0;
-  if (lane + 32 < p.out_channels) out[lane + 32] = res1;
 }
 
 __global__ void copy_out_kernel(const IoSlot* slot, const float* h, int64_t n4) {
@@ -691,16 +847,16 @@ __global__ void copy_out_kernel(const IoSlot* slot, const float* h, int64_t n4) 
     o[i] = s[i];
 }
 
-__global__ void pack_f16_kernel(f16* dst, int ld_dst, int col0, const float* h, int rows, int d) {
+// Thread (x, y): 8 columns of every gridDim.y-th row (d % 8 == 0).
+__global__ void __launch_bounds__(128) pack_f16_kernel(f16* dst, int ld_dst, int col0, const float* h, int rows, int d) {
   pdl_wait_and_trigger();
-  const int64_t n4 = static_cast<int64_t>(rows) * d / 4;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const int64_t e = i * 4;
-    const int64_t r = e / d;
-    const int c = static_cast<int>(e % d);
-    const float4 v = reinterpret_cast<const float4*>(h)[i];
-    store_f16x4(dst + r * ld_dst + col0 + c, v);
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) * 8;
+  if (c >= d) return;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+    const float4* src = reinterpret_cast<const float4*>(h + static_cast<int64_t>(r) * d + c);
+    const float4 a = src[0], b = src[1];
+    const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(r) * ld_dst + col0 + c) = pack_f16x8(f);
   }
 }
 
@@ -772,10 +928,28 @@ __global__ void rowdot_kernel(const TW* w, const bf16* x, int64_t rows, int K, f
   if (lane == 0) out[j] = static_cast<float>(acc * scale);
 }
 
-__global__ void sampler_kernel(float* z, const float* eps, float alpha, float beta, int64_t n) {
+// z and eps 16-byte aligned: 4 elements per thread and step, the rest by the first threads
+// (2.6 M elements: 8.1 us with one element per thread).
+__global__ void sampler_kernel(float* z, const float* eps, float alpha, float beta, int64_t n, int vec) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride)
-    z[i] = alpha * z[i] - beta * eps[i];
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  int64_t done = 0;
+  if (vec) {
+    const int64_t n4 = n >> 2;
+    float4* z4 = reinterpret_cast<float4*>(z);
+    const float4* e4 = reinterpret_cast<const float4*>(eps);
+    for (int64_t i = i0; i < n4; i += stride) {
+      float4 a = z4[i];
+      const float4 e = e4[i];
+      a.x = alpha * a.x - beta * e.x;
+      a.y = alpha * a.y - beta * e.y;
+      a.z = alpha * a.z - beta * e.z;
+      a.w = alpha * a.w - beta * e.w;
+      z4[i] = a;
+    }
+    done = n4 << 2;
+  }
+  for (int64_t i = done + i0; i < n; i += stride) z[i] = alpha * z[i] - beta * eps[i];
 }
 
 int grid_for(int64_t work, int threads) {
@@ -787,13 +961,27 @@ int grid_for(int64_t work, int threads) {
 
 }  // namespace
 
+namespace {
+template <int MODE>
+cudaError_t norm_launch_mode(const NormParams& p, cudaStream_t s) {
+  const dim3 grid((p.rows + 3) / 4), block(128);
+  if (p.d <= 256) return launch_k(norm_warp_kernel<2, MODE>, grid, block, 0, s, p);
+  if (p.d <= 512) return launch_k(norm_warp_kernel<4, MODE>, grid, block, 0, s, p);
+  if (p.d <= 1024) return launch_k(norm_warp_kernel<8, MODE>, grid, block, 0, s, p);
+  if (p.d <= 1280) return launch_k(norm_warp_kernel<10, MODE>, grid, block, 0, s, p);
+  if (p.d <= 2048) return launch_k(norm_warp_kernel<16, MODE>, grid, block, 0, s, p);
+  if (p.rows <= wide_blocks(false) * num_sms())
+    return launch_k(norm_wide_kernel<MODE, false>, dim3(p.rows), dim3(wide_threads(false)), 0, s, p);
+  return launch_k(norm_wide_kernel<MODE, true>, dim3(wide_blocks(true) * num_sms()), dim3(wide_threads(true)), 0, s, p);
+}
+}  // namespace
+
 cudaError_t norm_launch(const NormParams& p, cudaStream_t s) {
-  // warp per row up to d = 2048; wider rows (LLaDA's 4096) measured faster with the block
-  // per row (4.2 against 2.3 TB/s inside the step)
-  if (p.d <= 32 * 4 * kNormWarpMaxVec)
-    return launch_k(norm_warp_kernel, dim3((p.rows + 7) / 8), dim3(256), 0, s, p);
-  else
-    return launch_k(norm_kernel, dim3(p.rows), dim3(kNormThreads), 0, s, p);
+  if (!p.scale) return norm_launch_mode<kGain>(p, s);
+  // the modulation may lie at any float's address
+  const bool vec = p.ld_mod % 4 == 0 &&
+                   ((reinterpret_cast<uintptr_t>(p.shift) | reinterpret_cast<uintptr_t>(p.scale)) & 15u) == 0;
+  return vec && !p.g && !p.b ? norm_launch_mode<kMod>(p, s) : norm_launch_mode<kAny>(p, s);
 }
 
 cudaError_t wait_selftest_launch(int* status, int code, cudaStream_t s) {
@@ -818,57 +1006,69 @@ cudaError_t frozen_launch(const FrozenParams& p, cudaStream_t s) {
   return launch_k(frozen_kernel, dim3(grid_for(p.n / 8, 256)), dim3(256), 0, s, p);
 }
 
-cudaError_t io_set_launch(IoSlot* slot, const IoSlot& v, cudaStream_t s) {
-  io_set_kernel<<<1, 1, 0, s>>>(slot, v);
+cudaError_t io_set_launch(IoSlot* slot, const IoSlot& v, const TimeEmb& te, cudaStream_t s) {
+  io_set_kernel<<<std::max(1, (te.n + 31) / 32), 32, 0, s>>>(slot, v, te);
   return cudaGetLastError();
 }
 
 cudaError_t stem_launch(const StemParams& p, cudaStream_t s) {
-  if ((p.kind == SGD_STEM_PATCH || p.kind == SGD_STEM_PATCH_TOKENS) && p.d % 4 == 0 && p.d_in % 8 == 0 &&
-      p.d_in > 0) {
-    const int64_t total4 = static_cast<int64_t>(p.batch) * p.n_tokens * (p.d / 4);
-    return launch_k(stem_patch_kernel, dim3(static_cast<unsigned>((total4 + 255) / 256)), dim3(256), 0, s, p);
+  const int rows = p.batch * p.n_tokens;
+  if (p.kind != SGD_STEM_PATCH && p.kind != SGD_STEM_PATCH_TOKENS) {
+    // about 16 blocks of 128 threads per SM, as far as there are rows (d % 8 == 0, checked at creation)
+    const int gx = (p.d / 8 + 127) / 128;
+    const int gy = std::max(1, std::min(rows, 16 * num_sms() / gx));
+    return launch_k(stem_rows_kernel, dim3(gx, gy), dim3(128), 0, s, p);
   }
-  const int64_t total = static_cast<int64_t>(p.batch) * p.n_tokens * p.d;
+  const dim3 grid((p.d / 4 + 127) / 128, (rows + kPatchRows - 1) / kPatchRows);
+  if (p.d_in == 8) return launch_k(stem_patch_kernel<8>, grid, dim3(128), 0, s, p);
+  if (p.d_in == 16) return launch_k(stem_patch_kernel<16>, grid, dim3(128), 0, s, p);
+  if (p.d_in % 8 == 0) {
+    const int64_t total4 = static_cast<int64_t>(rows) * (p.d / 4);
+    return launch_k(stem_patch_any_kernel, dim3(static_cast<unsigned>((total4 + 255) / 256)), dim3(256), 0, s, p);
+  }
+  const int64_t total = static_cast<int64_t>(rows) * p.d;
   return launch_k(stem_kernel, dim3(static_cast<unsigned>((total + 255) / 256)), dim3(256), 0, s, p);
 }
 
-template <int RMAX>
+template <int RMAX, int COLS>
 cudaError_t gemv_launch_r(const GemvParams& p, size_t smem, cudaStream_t s) {
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(gemv_kernel<RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(gemv_kernel<RMAX, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
-  const int cols_per_block = 8 * kGemvCols;
+  const int cols_per_block = 8 * COLS;
   const int64_t items = static_cast<int64_t>((p.N + cols_per_block - 1) / cols_per_block) * (p.n_seg > 0 ? p.n_seg : 1);
   const int grid = static_cast<int>(std::min<int64_t>(items, 2 * static_cast<int64_t>(num_sms())));
-  return launch_k(gemv_kernel<RMAX>, dim3(grid), dim3(256), smem, s, p);
+  return launch_k(gemv_kernel<RMAX, COLS>, dim3(grid), dim3(256), smem, s, p);
 }
 
 cudaError_t gemv_launch(const GemvParams& p, cudaStream_t s) {
-  const int xrows = p.x_sinusoid ? 1 : (p.ldx == 0 ? 1 : p.rows);
+  const int xrows = p.ldx == 0 ? 1 : p.rows;
   const size_t smem = static_cast<size_t>(xrows) * p.K * sizeof(float);
   if (p.rows > 16 || smem > 200 * 1024 || (p.K % 8) || p.n_seg < 0 || p.n_seg > kGemvMaxSeg ||
       (p.n_seg > 0 && (p.out_silu || p.add_class || p.add_vec)) ||
-      (!p.x_sinusoid && ((p.ldx % 4) || (reinterpret_cast<uintptr_t>(p.x) & 15u))))
+      (p.ldx % 4) || (reinterpret_cast<uintptr_t>(p.x) & 15u))
     return cudaErrorInvalidValue;
-  if (xrows == 1) return gemv_launch_r<1>(p, smem, s);
-  if (xrows <= 8) return gemv_launch_r<8>(p, smem, s);
-  return gemv_launch_r<16>(p, smem, s);
+  if (xrows == 1) {
+    const bool few = static_cast<int64_t>(p.N) * std::max(p.n_seg, 1) < 64ll * num_sms();
+    return few ? gemv_launch_r<1, 1>(p, smem, s) : gemv_launch_r<1, 4>(p, smem, s);
+  }
+  if (xrows <= 8) return gemv_launch_r<8, 4>(p, smem, s);
+  return gemv_launch_r<16, 2>(p, smem, s);
 }
 
 cudaError_t head_small_launch(const HeadParams& p, cudaStream_t s) {
   const int64_t rows = static_cast<int64_t>(p.batch) * p.n_tokens;
-  const dim3 grid(static_cast<unsigned>((rows + 7) / 8));
   if (p.K % 4 || p.K > 4096 || p.out_channels > 64 || p.out_channels > p.N || p.ldx % 4 ||
       (p.shift && p.ld_mod % 4))
     return cudaErrorInvalidValue;
-  if (p.K <= 512) return launch_k(head_small_kernel<4>, grid, dim3(256), 0, s, p);
-  if (p.K <= 1024) return launch_k(head_small_kernel<8>, grid, dim3(256), 0, s, p);
-  if (p.K <= 1536) return launch_k(head_small_kernel<12>, grid, dim3(256), 0, s, p);
-  if (p.K <= 2048) return launch_k(head_small_kernel<16>, grid, dim3(256), 0, s, p);
-  return launch_k(head_small_kernel<32>, grid, dim3(256), 0, s, p);
+  const size_t smem = static_cast<size_t>(8) * p.K * sizeof(float);  // 4 warps of 2 rows: 128 KB at most
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(head_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
+  return launch_k(head_small_kernel, dim3(static_cast<unsigned>((rows + 7) / 8)), dim3(128), smem, s, p);
 }
 
 cudaError_t copy_out_launch(const IoSlot* slot, const float* h, int64_t n, cudaStream_t s) {
@@ -877,8 +1077,9 @@ cudaError_t copy_out_launch(const IoSlot* slot, const float* h, int64_t n, cudaS
 
 cudaError_t pack_f16_launch(f16* dst, int ld_dst, int col0, const float* h, int rows, int d,
                             cudaStream_t s) {
-  return launch_k(pack_f16_kernel, dim3(grid_for(static_cast<int64_t>(rows) * d / 4, 256)), dim3(256), 0, s,
-                  dst, ld_dst, col0, h, rows, d);
+  const int gx = (d / 8 + 127) / 128;
+  return launch_k(pack_f16_kernel, dim3(gx, std::max(1, std::min(rows, 16 * num_sms() / gx))), dim3(128), 0, s, dst,
+                  ld_dst, col0, h, rows, d);
 }
 
 cudaError_t absmax_bf16_launch(const bf16* w, int64_t n, float* out, cudaStream_t s) {
@@ -916,7 +1117,8 @@ cudaError_t rowdot_bf16_launch(const bf16* w, const bf16* x, int64_t rows, int K
 
 cudaError_t sampler_launch(float* z, const float* eps, float alpha, float beta, int64_t n,
                            cudaStream_t s) {
-  sampler_kernel<<<grid_for(n, 256), 256, 0, s>>>(z, eps, alpha, beta, n);
+  const int vec = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(eps)) & 15u) == 0 ? 1 : 0;
+  sampler_kernel<<<grid_for(vec ? (n + 3) / 4 : n, 256), 256, 0, s>>>(z, eps, alpha, beta, n, vec);
   return cudaGetLastError();
 }
 

@@ -210,7 +210,13 @@ struct IoSlot {
   float t;
   int step;
 };
-cudaError_t io_set_launch(IoSlot* slot, const IoSlot& v, cudaStream_t s);
+// Time embeddings of a step: n values, the first dim0 of one width, the rest of another.
+struct TimeEmb {
+  float* out = nullptr;
+  const double* w = nullptr;  // frequencies: dim0 / 2, then (n - dim0) / 2
+  int n = 0, dim0 = 0;
+};
+cudaError_t io_set_launch(IoSlot* slot, const IoSlot& v, const TimeEmb& te, cudaStream_t s);
 
 // Small always-on pieces (stem, conditioning, heads).
 struct StemParams {
@@ -222,18 +228,18 @@ struct StemParams {
   const bf16* pos;
   const bf16* class_emb;
   const bf16* embed;
+  const float* time;    // the step's time embedding [d] (TimeEmb)
   int vocab, n_classes;  // ids are clamped into [0, vocab) / [0, n_classes)
 };
 cudaError_t stem_launch(const StemParams& p, cudaStream_t s);
 
-// out[r, j] = sum_k act(x[r, k]) W[j, k] (+ add[r, j]); x fp32 or computed on the fly.
+// out[r, j] = sum_k act(x[r, k]) W[j, k] (+ add[r, j]); x fp32.
 constexpr int kGemvMaxSeg = 64;
 struct GemvParams {
   float* out;
   int ldo;
-  const float* x;      // [rows, K] fp32 (ignored when x_sinusoid)
-  int ldx;
-  int x_sinusoid;      // x = sinusoid(t, K) from the slot, one row
+  const float* x;      // [rows, K] fp32
+  int ldx;             // 0: one row, used for every output row
   const IoSlot* slot;
   int in_silu;         // act = silu
   const bf16* W;       // [N, K]
