@@ -102,21 +102,22 @@ SGD_API int sgd_kernel_gemm_stat_slots(int M, int N, int K, const sgd_epilogue_a
 /*
  * C = alpha A B^T.  A fp16 [M, K] (row stride lda elements), B fp16 [N or 2N, K]
  * (row stride ldb).  K, lda, ldb multiples of 8; N multiple of 8; pointers 16-byte
- * aligned.  use_simt = 1 runs the plain SIMT kernel (reference / debugging), 0 a
- * tcgen05 + TMA kernel (fp32 accumulators in TMEM) with 64-element K-blocks: where M > 128
- * and its tiles fit at least as well, the CTA-pair kernel (256 x 128 .. 256 x 256 tiles, M = 256
- * instructions over two SMs), otherwise the one-CTA kernel (M = 128, N = 256, K = 16
- * instructions), choosing by itself 128 x 256 or 128 x 128 tiles, 4 or 8
+ * aligned.  use_simt = 1 runs the plain SIMT kernel (reference / debugging); the others are
+ * tcgen05 + TMA kernels (fp32 accumulators in TMEM).  0 runs the CTA-group kernel, whose tiles of
+ * 128 x 64 to 128 x 256 (one CTA) or 256 x 128 to 256 x 256 (a cluster of two CTAs, M = 256
+ * instructions; M > 128) it chooses by their cost.  With a folded norm or the residual writer
+ * below, and in the forms 3 and 5 to 12, the one-CTA kernel (M = 128, N = 256, K = 16
+ * instructions, 64-element K-blocks) runs, choosing by itself 128 x 256 or 128 x 128 tiles, 4 or 8
  * epilogue warps, and whether the tiles left over after the last full wave of CTAs are
  * split along K over all SMs ("stream-K": fp32 partial tiles in a workspace, summed in a
- * fixed order by the CTA that finishes a tile last, so results are deterministic); 3 the
- * form of 0 with 32-element K-blocks (64-byte swizzle); 2 and 4 are not defined and are
- * rejected with SGD_ERR_ARG; 3 and 5 to 12 are forms of the one-CTA kernel: 5, 6, 7 force 128 x 256 tiles with 4 epilogue warps, 128 x 256 with 8, and
+ * fixed order by the CTA that finishes a tile last, so results are deterministic).  3: with
+ * 32-element K-blocks (64-byte swizzle); 2 and 4 are not defined and are
+ * rejected with SGD_ERR_ARG; 5, 6, 7 force 128 x 256 tiles with 4 epilogue warps, 128 x 256 with 8, and
  * 128 x 128 with 8 and no stream-K (128 x 128 applies to plain, GELU and DELTA epilogues
- * only); 8 is 0 without stream-K, 9 is 0 with stream-K whenever the last wave is partial;
+ * only); 8 is without stream-K, 9 with stream-K whenever the last wave is partial;
  * 10 forces 128 x 224 tiles (5 pipeline stages, no stream-K; plain, GELU and DELTA only);
- * 11 and 12 are 0 with the tiles visited M-fastest, and in groups of 16 row-blocks (each
- * group column by column, every other group backwards), instead of the choice made by 0
+ * 11 and 12 have the tiles visited M-fastest, and in groups of 16 row-blocks (each
+ * group column by column, every other group backwards), instead of by choice
  * (groups where there are at least two groups and two waves).
  * The stream-K workspace is owned by the library, one per (device, stream), allocated
  * or grown by the first call that needs it (after synchronising that stream).

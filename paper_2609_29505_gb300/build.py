@@ -19,8 +19,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsgd.so")
 
-SOURCES = ["gemm_tc_plain.cu", "gemm_tc_rms.cu", "gemm_tc_ln.cu", "gemm_tc_h16.cu", "gemm_pair_delta.cu",
-           "gemm_pair_plain.cu", "gemm_pair_act.cu", "gemm.cu",
+SOURCES = ["gemm_tc_plain.cu", "gemm_tc_rms.cu", "gemm_tc_ln.cu", "gemm_tc_h16.cu", "gemm_group_delta.cu",
+           "gemm_group_plain.cu", "gemm_group_act.cu", "gemm.cu",
            "attention.cu", "elementwise.cu", "api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fno-strict-aliasing",

@@ -308,13 +308,13 @@ int make_gemm_op(sgd_ctx* c, std::vector<Op>& ops, const std::string& name, cons
   plan->epi = epi;
   plan->simt = (c->d.flags & SGD_FLAG_SIMT_GEMM) != 0;
   plan->bk = (c->d.flags & SGD_FLAG_GEMM_BK64) ? 64 : c->gemm_bk;
-  plan->allow_pair = true;
+  plan->allow_group = true;
   const char* why = "";
   if (gemm_plan(*plan, &why) != 0) return fail(SGD_ERR_SHAPE, std::string(name) + ": " + why);
   plan->ws_ref = &c->sk_ws;
   plan->cnt_ref = &c->sk_cnt;
   c->sk_need_floats = std::max(c->sk_need_floats, gemm_ws_floats(*plan));
-  c->sk_need_cnt = std::max(c->sk_need_cnt, gemm_ws_tickets(*plan));
+  c->sk_need_cnt = std::max(c->sk_need_cnt, plan->sk_tiles);
   const bool gated = epi.kind == SGD_EPI_GATED;
   const double nb = gated ? 2.0 * N : N;
   double out_b;
@@ -1759,7 +1759,7 @@ int kernel_gemm_plan(const void* A, int lda, const void* B, int ldb, int M, int 
   p.N = N;
   p.K = K;
   p.simt = variant == 1;
-  p.allow_pair = p.encode && variant == 0;  // (the statistics slots are those of the one-CTA kernel)
+  p.allow_group = p.encode && variant == 0;  // (the statistics slots are those of the one-CTA kernel)
   p.bk = variant == 3 ? 32 : 64;
   if (variant == 5) { p.bn = 256; p.epiw = 4; }
   if (variant == 6) { p.bn = 256; p.epiw = 8; }
@@ -1820,12 +1820,12 @@ int sgd_kernel_gemm(const void* A, int lda, const void* B, int ldb, int M, int N
     int dev = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     KernelWs* w = nullptr;
-    const int wrc = kernel_ws(dev, stream, gemm_ws_floats(p), gemm_ws_tickets(p), &w);
+    const int wrc = kernel_ws(dev, stream, gemm_ws_floats(p), p.sk_tiles, &w);
     if (wrc) return wrc;
     p.ws_ref = &w->ws;
     p.cnt_ref = &w->cnt;
     // a launch that stopped on an expired wait can leave counters behind; start from zero
-    CUDA_TRY(cudaMemsetAsync(w->cnt, 0, sizeof(int) * gemm_ws_tickets(p), static_cast<cudaStream_t>(stream)));
+    CUDA_TRY(cudaMemsetAsync(w->cnt, 0, sizeof(int) * p.sk_tiles, static_cast<cudaStream_t>(stream)));
   }
   CUDA_TRY(gemm_launch(p, static_cast<cudaStream_t>(stream)));
   return SGD_OK;
@@ -1839,13 +1839,13 @@ int sgd_kernel_gemm_static_ws(const void* A, int lda, const void* B, int ldb, in
   const char* why = "";
   float* ws = nullptr;
   int* tickets = nullptr;
-  if (p.pair) {
+  if (p.group) {
     // the entry's size limit is that of the one-CTA kernel's split, whichever kernel runs
     GemmPlan q = p;
-    q.allow_pair = q.encode = false;
+    q.allow_group = q.encode = false;
     q.bn = q.epiw = 0;
     q.sk = q.group_m = -1;
-    if (gemm_plan(q, &why) == 0 && q.sk_tiles > 0 && gemm_ws_floats(q) * sizeof(float) > gemm_static_ws_bytes())
+    if (gemm_plan(q, &why) == 0 && gemm_ws_floats(q) * sizeof(float) > gemm_static_ws_bytes())
       return fail(SGD_ERR_SHAPE, "gemm: the stream-K split of this problem needs more than the static scratch "
                                  "(use sgd_kernel_gemm, or variant 8)");
   }
@@ -1853,7 +1853,7 @@ int sgd_kernel_gemm_static_ws(const void* A, int lda, const void* B, int ldb, in
     size_t cap = 0;
     int n_cap = 0;
     if (gemm_static_scratch(&ws, &cap, &tickets, &n_cap, &why)) return fail(SGD_ERR_CUDA, why);
-    if (gemm_ws_floats(p) > cap || gemm_ws_tickets(p) > n_cap)
+    if (gemm_ws_floats(p) > cap || p.sk_tiles > n_cap)
       return fail(SGD_ERR_SHAPE, "gemm: the stream-K split of this problem needs " +
                                      std::to_string(gemm_ws_floats(p) * sizeof(float)) +
                                      " bytes of partial tiles, more than the " + std::to_string(cap * sizeof(float)) +
@@ -1861,7 +1861,7 @@ int sgd_kernel_gemm_static_ws(const void* A, int lda, const void* B, int ldb, in
     p.ws_ref = &ws;
     p.cnt_ref = &tickets;
     // the tickets must start at zero (a launch stopped on an expired wait can leave some)
-    CUDA_TRY(cudaMemsetAsync(tickets, 0, sizeof(int) * gemm_ws_tickets(p), static_cast<cudaStream_t>(stream)));
+    CUDA_TRY(cudaMemsetAsync(tickets, 0, sizeof(int) * p.sk_tiles, static_cast<cudaStream_t>(stream)));
   }
   CUDA_TRY(gemm_launch(p, static_cast<cudaStream_t>(stream)));
   return SGD_OK;

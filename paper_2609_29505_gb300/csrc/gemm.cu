@@ -3,11 +3,12 @@
 // word and the fixed scratch of the allocation-free entry.  The kernel itself is in
 // gemm_kernel.cuh.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
 
-#include "gemm_pair_kernel.cuh"
+#include "gemm_group_kernel.cuh"
 
 namespace sgd {
 
@@ -28,22 +29,32 @@ SGD_GEMM_EXTERN(kFeatRms)
 SGD_GEMM_EXTERN(kFeatLn)
 SGD_GEMM_EXTERN(kFeatH16)
 #undef SGD_GEMM_EXTERN
-#define SGD_PAIR_EXTERN(BN, EP) \
-  extern template cudaError_t launch_pair<BN, EP>(const GemmPlan&, const TcArgs&, cudaStream_t);
-SGD_PAIR_EXTERN(256, kEpDelta)
-SGD_PAIR_EXTERN(224, kEpDelta)
-SGD_PAIR_EXTERN(192, kEpDelta)
-SGD_PAIR_EXTERN(160, kEpDelta)
-SGD_PAIR_EXTERN(128, kEpDelta)
-SGD_PAIR_EXTERN(256, kEpPlain)
-SGD_PAIR_EXTERN(224, kEpPlain)
-SGD_PAIR_EXTERN(192, kEpPlain)
-SGD_PAIR_EXTERN(160, kEpPlain)
-SGD_PAIR_EXTERN(128, kEpPlain)
-SGD_PAIR_EXTERN(256, kEpGated)
-SGD_PAIR_EXTERN(224, kEpGated)
-SGD_PAIR_EXTERN(256, kEpRope)
-#undef SGD_PAIR_EXTERN
+#define SGD_GROUP_EXTERN(CG, BN, EP) \
+  extern template cudaError_t launch_group<CG, BN, EP>(const GemmPlan&, const TcArgs&, cudaStream_t);
+SGD_GROUP_EXTERN(2, 256, kEpDelta)
+SGD_GROUP_EXTERN(2, 224, kEpDelta)
+SGD_GROUP_EXTERN(2, 192, kEpDelta)
+SGD_GROUP_EXTERN(2, 160, kEpDelta)
+SGD_GROUP_EXTERN(2, 128, kEpDelta)
+SGD_GROUP_EXTERN(1, 256, kEpDelta)
+SGD_GROUP_EXTERN(1, 128, kEpDelta)
+SGD_GROUP_EXTERN(1, 64, kEpDelta)
+SGD_GROUP_EXTERN(2, 256, kEpPlain)
+SGD_GROUP_EXTERN(2, 224, kEpPlain)
+SGD_GROUP_EXTERN(2, 192, kEpPlain)
+SGD_GROUP_EXTERN(2, 160, kEpPlain)
+SGD_GROUP_EXTERN(2, 128, kEpPlain)
+SGD_GROUP_EXTERN(1, 256, kEpPlain)
+SGD_GROUP_EXTERN(1, 128, kEpPlain)
+SGD_GROUP_EXTERN(1, 64, kEpPlain)
+SGD_GROUP_EXTERN(2, 256, kEpGated)
+SGD_GROUP_EXTERN(2, 224, kEpGated)
+SGD_GROUP_EXTERN(1, 256, kEpGated)
+SGD_GROUP_EXTERN(1, 128, kEpGated)
+SGD_GROUP_EXTERN(2, 256, kEpRope)
+SGD_GROUP_EXTERN(1, 256, kEpRope)
+SGD_GROUP_EXTERN(1, 128, kEpRope)
+#undef SGD_GROUP_EXTERN
 }  // namespace gk
 
 namespace {
@@ -266,49 +277,47 @@ SkSplit sk_split(int num_tiles, int num_k, int sms, bool force = false) {
   return r;
 }
 
-// Whether the CTA-pair kernel runs this problem, and its tile width (sets p.pair, p.bn).
-// A launch takes about waves x K-blocks x the time of a K-block, something for every wave, and
-// the last tile's epilogue.  A K-block takes the tensor cores 2 BN clocks, unless its operand
-// bytes take longer to reach the SM (73 to 79 per clock with all SMs loading); the constants are
-// fitted to graph-replayed launches of 36 shapes, where the chosen width was within 4% of the best
-// (us, one-CTA kernel / widths 128, 160, 192, 224, 256):
-//   2048 x 1152 x 4608 residual  24.3 / 21.4  23.6  25.6  28.4  31.1
-//   2048 x 1280 x 5120 residual  38.7 / 36.7  25.3  27.7  30.3  33.6
-//   2048 x 3456 x 1152 fp16      20.5 / 17.8  18.7  16.2  17.3  18.1
-//   4096 x 4096 x 4096 residual 104.0 / 98.5  94.8  93.6  87.4  93.7
-//   4096 x 12288 x 4096 fp16    290.8 / 294.8 251.9 226.0 220.8 234.0
-//   333 x 12288 x 4096 gated     66.3 /  -     -     -    71.0  79.2
+// Tile of the CTA-group kernel (sets p.group, p.bn).  In SM clocks, a launch takes about
+//   waves x (K-blocks x time of a K-block + kWave) + the last tile's epilogue (+ kPair),
+// a K-block a little over 2 BN on the tensor cores, or the issue loop's 324, unless its operand
+// bytes take longer to reach the SM (kRate per clock with all SMs loading).  The constants are
+// fitted to graph-replayed launches of 46 shapes, of which the chosen tile is within 5% of the best
+// (us; a CTA's 128 x 64, 128, 256 / a pair's 256 x 128, 160, 192, 224, 256):
+//   64 x 256 x 256 residual       4.7   5.8   9.1 /
+//   300 x 520 x 688 fp16          5.6   6.8   9.3 /  7.4   7.6   8.1   8.8   9.1
+//   2048 x 1152 x 1152 residual  11.1  10.1  15.2 / 10.9  12.2  12.2  13.7  15.6
+//   2048 x 1152 x 4608 residual  30.1  22.8  34.8 / 22.0  23.8  25.7  28.3  31.2
+//   2048 x 1280 x 5120 residual  45.6  38.5  37.7 / 36.9  25.4  27.6  30.3  33.5
+//   2048 x 3456 x 1152 fp16      24.9  17.8  19.4 / 17.5  18.8  15.9  17.6  18.3
+//   4096 x 4096 x 4096 residual   161   109   111 / 99.5  99.3  99.1  92.6 102.3
+//   333 x 12288 x 4096 RoPE       -    42.4  42.1 /  -     -     -     -    60.5
 // The last one has 333 rows: 512 in 256-row tiles, 384 in 128-row ones.  At M <= 128 half of
 // every pair would compute rows that do not exist.
-void plan_pair(GemmPlan& p, int sms) {
+void plan_group(GemmPlan& p, int sms) {
   const EpiParams& e = p.epi;
   const bool gated = e.kind == SGD_EPI_GATED, rope = e.kind == SGD_EPI_ROPE;
-  const int pairs = sms / 2;
-  if (p.M <= kBM || pairs < 1) return;
-  constexpr double kPairBytes = 73.0, kOneBytes = 79.0, kWave = 1300.0;
   const double epi_col = e.kind == SGD_EPI_DELTA ? 40.0 : 25.0;
   const int num_k = (p.K + 63) / 64;
-  auto cost = [&](int rows, int bn, int b_rows, int workers, double bytes_per_clk) {
-    const int cols = gated ? bn / 2 : bn;
-    const int tiles = ((p.M + rows - 1) / rows) * ((p.N + cols - 1) / cols);
-    const double block = std::max(2.0 * bn, 128.0 * (kBM + b_rows) / bytes_per_clk);
-    return ((tiles + workers - 1) / workers) * (num_k * block + kWave) + epi_col * bn;
-  };
-  double one = cost(kBM, 256, 256, sms, kOneBytes);
-  if (!gated && !rope) one = std::min(one, cost(kBM, 128, 128, sms, kOneBytes));
+  struct Tile { int cg, bn; };
+  static const Tile kTiles[] = {{2, 256}, {2, 224}, {2, 192}, {2, 160}, {2, 128}, {1, 256}, {1, 128}, {1, 64}};
   double best = 0;
-  int best_bn = 0;
-  for (int bn : {256, 224, 192, 160, 128}) {
-    if ((gated && bn < 224) || (rope && bn != 256)) continue;
-    const double c = cost(2 * kBM, bn, bn / 2, pairs, kPairBytes);
-    if (best_bn == 0 || c < best) {
-      best = c;
-      best_bn = bn;
+  for (const Tile& t : kTiles) {
+    const bool pair = t.cg == 2;
+    const int workers = sms / t.cg, cols = gated ? t.bn / 2 : t.bn;
+    if (workers < 1 || (pair && p.M <= kBM)) continue;
+    if (gated && t.bn < (pair ? 224 : 128)) continue;
+    if (rope && t.bn < (pair ? 256 : 128)) continue;
+    const double kRate = pair ? 62.0 : 71.0, kWave = pair ? 1300.0 : 600.0, kPair = pair ? 2700.0 : 0.0;
+    const double rows = t.cg * kBM;
+    const double tiles = std::ceil(p.M / rows) * std::ceil(static_cast<double>(p.N) / cols);
+    const double block = std::max({2.06 * t.bn, 324.0, 128.0 * (kBM + t.bn / t.cg) / kRate});
+    const double cost = std::ceil(tiles / workers) * (num_k * block + kWave) + epi_col * t.bn + kPair;
+    if (best == 0 || cost < best) {
+      best = cost;
+      p.group = t.cg;
+      p.bn = t.bn;
     }
   }
-  if (one < 0.98 * best) return;
-  p.pair = true;
-  p.bn = best_bn;
 }
 
 int gemm_plan(GemmPlan& p, const char** why) {
@@ -390,11 +399,12 @@ int gemm_plan(GemmPlan& p, const char** why) {
   const int b_rows = gated ? 2 * p.N : p.N;
   if (p.bk != 64 && p.bk != 32) p.bk = 64;
   const int sms = num_sms();
-  p.pair = false;
-  if (p.allow_pair && p.bk == 64 && p.bn == 0 && p.epiw == 0 && p.sk == -1 && p.group_m < 0 &&
+  p.group = 0;
+  if (p.allow_group && p.bk == 64 && p.bn == 0 && p.epiw == 0 && p.sk == -1 && p.group_m < 0 &&
       e.norm == SGD_FNORM_NONE && !e.h16)
-    plan_pair(p, sms);
-  const int num_m = p.pair ? (p.M + 2 * kBM - 1) / (2 * kBM) : (p.M + kBM - 1) / kBM;
+    plan_group(p, sms);
+  const int rows = (p.group ? p.group : 1) * kBM;
+  const int num_m = (p.M + rows - 1) / rows;
   const int num_k = (p.K + p.bk - 1) / p.bk;
   // tile shape: 128-column tiles when they need clearly fewer tile-times than 256-column
   // tiles (a 128-column tile takes half the time of a 256-column one, at about 3/4 of its
@@ -405,7 +415,7 @@ int gemm_plan(GemmPlan& p, const char** why) {
   // tiles wastes under a tenth of N (e.g. M = N = 4096 at K >= 3072: 608 tiles = 4 waves;
   // measured 1266 against 1233 TFLOP/s for 128 x 256 with stream-K)
   const int n224 = (p.N + 223) / 224;
-  if (!p.pair && p.bn == 0 && p.sk != 1 && small_ok && p.K >= 3072 && (num_m * n224) % sms == 0 &&
+  if (!p.group && p.bn == 0 && p.sk != 1 && small_ok && p.K >= 3072 && (num_m * n224) % sms == 0 &&
       10 * (n224 * 224 - p.N) < p.N)
     p.bn = 224;
   if (p.bn == 0) {
@@ -416,8 +426,8 @@ int gemm_plan(GemmPlan& p, const char** why) {
     const bool sk_on = p.sk != 0 && sk256.tiles > 0;
     p.bn = (small_ok && !sk_on && 2 * w128 < 3 * w256) ? 128 : 256;
   }
-  if (!p.pair && ((p.bn != 128 && p.bn != 224) || !small_ok)) p.bn = 256;
-  if (p.bn == 224) p.sk = 0;
+  if (!p.group && ((p.bn != 128 && p.bn != 224) || !small_ok)) p.bn = 256;
+  if (!p.group && p.bn == 224) p.sk = 0;
   // 8 epilogue warps (two per TMEM lane quarter, staged stores) except for RoPE, whose
   // per-thread state needs the 4-warp kernel's registers, and long-K gated MLPs, whose
   // epilogue hides behind the main loop (device time per launch: gated 2048 x 5120 x 1280
@@ -425,8 +435,10 @@ int gemm_plan(GemmPlan& p, const char** why) {
   // 4096 x 12288 x 4096 259 against 305 us with 8)
   if (p.epiw == 0) p.epiw = (e.kind == SGD_EPI_ROPE || (gated && p.K >= 3072)) ? 4 : 8;
   if (p.bn == 128 || p.bn == 224 || p.bk == 32) p.epiw = 8;
+  // rows of B per load: the group kernel takes its whole part of B (gated: one of two) at once
+  const int box_b = p.group ? ((p.group == 2 || gated) ? p.bn / 2 : p.bn) : (p.bn == 224 ? 224 : 128);
   if (p.encode && (!make_tmap_f16(&p.tmap_a, p.A, p.M, p.K, p.lda, 128, p.bk) ||
-                   !make_tmap_f16(&p.tmap_b, p.B, b_rows, p.K, p.ldb, p.pair ? p.bn / 2 : (p.bn == 224 ? 224 : 128), p.bk))) {
+                   !make_tmap_f16(&p.tmap_b, p.B, b_rows, p.K, p.ldb, box_b, p.bk))) {
     *why = "gemm: cuTensorMapEncodeTiled failed (driver entry point unavailable or bad layout)";
     return -5;
   }
@@ -436,7 +448,8 @@ int gemm_plan(GemmPlan& p, const char** why) {
     return -2;
   }
   const int units = num_m * num_n;
-  p.grid = p.pair ? 2 * std::min(units, sms / 2) : std::min(units, sms);
+  p.grid = std::min(units, sms);
+  if (p.group) p.grid = p.group * std::min(units, sms / p.group);
   // tile order.  M-fastest keeps A (the activations) in L2 while B streams through once,
   // which is the least DRAM traffic whenever A fits in L2 with room to spare (QKV, up, head
   // and attention-output projections: A = 33.5 MB).  When neither operand fits (the down
@@ -445,14 +458,14 @@ int gemm_plan(GemmPlan& p, const char** why) {
   if (p.group_m < 0) {
     const double a_bytes = 2.0 * p.M * p.K, b_bytes = 2.0 * b_rows * p.K;
     constexpr double kL2Resident = 48e6;  // of 129 MB of L2, split between two dies
-    const int m128 = p.pair ? 2 * num_m : num_m, tiles128 = p.pair ? 2 * units : units;
+    const int m128 = p.group == 2 ? 2 * num_m : num_m, tiles128 = p.group == 2 ? 2 * units : units;
     p.group_m = (m128 >= 32 && num_n >= 4 && tiles128 >= 2 * sms && a_bytes > kL2Resident &&
                  b_bytes > kL2Resident)
-                    ? (p.pair ? 8 : 16)
+                    ? (p.group == 2 ? 8 : 16)
                     : 0;
   }
   p.sk_tiles = p.sk_ctas = p.max_seg = 0;
-  if (p.sk != 0 && !p.pair) {
+  if (p.sk != 0 && !p.group) {
     const SkSplit k = sk_split(units, num_k, sms, p.sk == 1);
     if (k.tiles > 0) {
       p.sk_tiles = k.tiles;
@@ -465,10 +478,9 @@ int gemm_plan(GemmPlan& p, const char** why) {
 }
 
 size_t gemm_ws_floats(const GemmPlan& p) {
-  return p.sk_tiles > 0 ? static_cast<size_t>(gemm_ws_tickets(p)) * p.max_seg * kBM * p.bn : 0;
+  return p.sk_tiles > 0 ? static_cast<size_t>(p.sk_tiles) * p.max_seg * kBM * p.bn : 0;
 }
 
-int gemm_ws_tickets(const GemmPlan& p) { return p.pair ? 2 * p.sk_tiles : p.sk_tiles; }
 
 template <int FEAT>
 cudaError_t launch_feat(const GemmPlan& p, const TcArgs& a, cudaStream_t s) {
@@ -479,22 +491,30 @@ cudaError_t launch_feat(const GemmPlan& p, const TcArgs& a, cudaStream_t s) {
 }
 
 template <int EP>
-cudaError_t launch_pair_bn(const GemmPlan& p, const TcArgs& a, cudaStream_t s) {
+cudaError_t launch_group_bn(const GemmPlan& p, const TcArgs& a, cudaStream_t s) {
+  if (p.group == 1) {
+    if (p.bn == 64) return launch_group<1, 64, EP>(p, a, s);
+    return p.bn == 128 ? launch_group<1, 128, EP>(p, a, s) : launch_group<1, 256, EP>(p, a, s);
+  }
   switch (p.bn) {
-    case 224: return launch_pair<224, EP>(p, a, s);
-    case 192: return launch_pair<192, EP>(p, a, s);
-    case 160: return launch_pair<160, EP>(p, a, s);
-    case 128: return launch_pair<128, EP>(p, a, s);
-    default: return launch_pair<256, EP>(p, a, s);
+    case 224: return launch_group<2, 224, EP>(p, a, s);
+    case 192: return launch_group<2, 192, EP>(p, a, s);
+    case 160: return launch_group<2, 160, EP>(p, a, s);
+    case 128: return launch_group<2, 128, EP>(p, a, s);
+    default: return launch_group<2, 256, EP>(p, a, s);
   }
 }
 
-cudaError_t launch_pair_any(const GemmPlan& p, const TcArgs& a, cudaStream_t s) {
+cudaError_t launch_group_any(const GemmPlan& p, const TcArgs& a, cudaStream_t s) {
   switch (p.epi.kind) {
-    case SGD_EPI_DELTA: return launch_pair_bn<kEpDelta>(p, a, s);
-    case SGD_EPI_GATED: return p.bn == 224 ? launch_pair<224, kEpGated>(p, a, s) : launch_pair<256, kEpGated>(p, a, s);
-    case SGD_EPI_ROPE: return launch_pair<256, kEpRope>(p, a, s);
-    default: return launch_pair_bn<kEpPlain>(p, a, s);
+    case SGD_EPI_DELTA: return launch_group_bn<kEpDelta>(p, a, s);
+    case SGD_EPI_GATED:
+      if (p.group == 2) return p.bn == 224 ? launch_group<2, 224, kEpGated>(p, a, s) : launch_group<2, 256, kEpGated>(p, a, s);
+      return p.bn == 128 ? launch_group<1, 128, kEpGated>(p, a, s) : launch_group<1, 256, kEpGated>(p, a, s);
+    case SGD_EPI_ROPE:
+      if (p.group == 2) return launch_group<2, 256, kEpRope>(p, a, s);
+      return p.bn == 128 ? launch_group<1, 128, kEpRope>(p, a, s) : launch_group<1, 256, kEpRope>(p, a, s);
+    default: return launch_group_bn<kEpPlain>(p, a, s);
   }
 }
 
@@ -514,7 +534,8 @@ cudaError_t gemm_launch(const GemmPlan& p, cudaStream_t s) {
   a.N = p.N;
   a.K = p.K;
   a.gated = p.epi.kind == SGD_EPI_GATED;
-  a.num_m = p.pair ? (p.M + 2 * kBM - 1) / (2 * kBM) : (p.M + kBM - 1) / kBM;
+  const int rows = (p.group ? p.group : 1) * kBM;
+  a.num_m = (p.M + rows - 1) / rows;
   a.num_n = a.gated ? (p.N + p.bn / 2 - 1) / (p.bn / 2) : (p.N + p.bn - 1) / p.bn;
   a.num_k = (p.K + p.bk - 1) / p.bk;
   a.group_m = p.group_m;
@@ -525,7 +546,7 @@ cudaError_t gemm_launch(const GemmPlan& p, cudaStream_t s) {
   a.ws = p.ws_ref ? *p.ws_ref : nullptr;
   a.sk_cnt = p.cnt_ref ? *p.cnt_ref : nullptr;
   if (p.sk_tiles > 0 && (!a.ws || !a.sk_cnt)) return cudaErrorInvalidValue;
-  if (p.pair) return launch_pair_any(p, a, s);
+  if (p.group) return launch_group_any(p, a, s);
   const EpiParams& e = p.epi;
   const int feat = e.norm == SGD_FNORM_RMS ? kFeatRms
                    : (e.norm == SGD_FNORM_LN ? kFeatLn : (e.h16 ? kFeatH16 : kFeatPlain));

@@ -340,9 +340,9 @@ __device__ __forceinline__ void emit_stats(const EpiParams& e, int row, int slot
 // free of bank conflicts).  Per 32-column chunk each thread puts its row's accumulator in
 // shared memory, and the warp then reads, updates and stores h and the fp16 cache with 8 lanes
 // per 128-byte row segment (with one thread per row the same accesses touch 32 rows per
-// instruction).  h does not depend on the accumulator: load_h_chunk fetches the first chunk
-// before the wait for it, and every further chunk while the one before is added, so that no
-// global load latency is left between the last MMA and the last store.
+// instruction).  h does not depend on the accumulator: with kAhead, load_h_chunk fetches the first
+// chunk before the wait for it, and every further chunk while the one before is added, so that
+// no global load latency is left between the last MMA and the last store.
 __device__ __forceinline__ void load_h_chunk(const TcArgs& a, int row0, int col0, float4* hv) {
   const int lane = threadIdx.x & 31;
   const int lr = lane >> 3, col = col0 + 4 * (lane & 7);
@@ -355,8 +355,8 @@ __device__ __forceinline__ void load_h_chunk(const TcArgs& a, int row0, int col0
   }
 }
 
-// kAhead: hv holds the first chunk of h (otherwise, for stream-K partial sums, whose source
-// needs the registers, each chunk is loaded where it is used).
+// kAhead: hv holds the first chunk of h (otherwise, in the one-CTA kernel, which has no
+// registers to spare for it, each chunk is loaded where it is used).
 template <bool kAhead, class Src>
 __device__ __forceinline__ void delta_staged(const TcArgs& a, int row, int n0, const Src& src, int cb, int ce,
                                              float4* stg, float4* hv) {
@@ -473,7 +473,7 @@ __device__ __forceinline__ void stage_flush_f32(const EpiParams& e, void* out, i
 template <int BN, bool kFastRope, int FEAT, class Src>
 __device__ __forceinline__ void epilogue_tile(const TcArgs& a, void* out, int row, int n_blk,
                                               const Src& src, int cb, int ce, int part, int halves,
-                                              float4* stg, float4* hv) {
+                                              float4* stg) {
   constexpr int kBN = BN;
   constexpr bool kH16 = FEAT == kFeatH16;
   // compile-time pruning of paths a feature set never takes (gemm_plan enforces it): a
@@ -611,7 +611,7 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& a, void* out, int ro
   if (!kNormFeat && e.kind == SGD_EPI_DELTA) {
     if constexpr (!kH16 && !kFastRope) {  // 8-warp kernels (the 4-warp RoPE kernel has no registers to spare)
       if (stg != nullptr) {
-        delta_staged<std::is_same<Src, TmemSrc>::value>(a, row, n0, src, cb, ce, stg, hv);
+        delta_staged<false>(a, row, n0, src, cb, ce, stg, nullptr);
         return;
       }
     }
@@ -799,16 +799,15 @@ struct CtaWork {
   int unit0, unit_step, n_units;
 };
 
-// `worker`: the CTA's (or CTA pair's) index among the sk_ctas of the stream-K split.
-__device__ __forceinline__ CtaWork cta_work(const TcArgs& a, int num_tiles, int unit0, int unit_step, int worker) {
+__device__ __forceinline__ CtaWork cta_work(const TcArgs& a, int num_tiles, int unit0, int unit_step) {
   CtaWork w;
   w.unit0 = unit0;
   w.unit_step = unit_step;
   w.sk_s = w.sk_e = w.t_sk0 = w.n_sk = 0;
-  if (a.sk_tiles > 0 && worker < a.sk_ctas) {
+  if (a.sk_tiles > 0 && static_cast<int>(blockIdx.x) < a.sk_ctas) {
     const int total = a.sk_tiles * a.num_k;
-    w.sk_s = sk_start(worker, total, a.sk_ctas);
-    w.sk_e = sk_start(worker + 1, total, a.sk_ctas);
+    w.sk_s = sk_start(blockIdx.x, total, a.sk_ctas);
+    w.sk_e = sk_start(blockIdx.x + 1, total, a.sk_ctas);
     w.t_sk0 = w.sk_s / a.num_k;
     w.n_sk = (w.sk_e - 1) / a.num_k - w.t_sk0 + 1;
   }
@@ -924,7 +923,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
   const uint32_t tmem_base = *tmem_slot;
   const int num_mu = a.num_m;
   const int num_tiles = num_mu * a.num_n;
-  const CtaWork w = cta_work(a, num_tiles, blockIdx.x, gridDim.x, blockIdx.x);
+  const CtaWork w = cta_work(a, num_tiles, blockIdx.x, gridDim.x);
 
   if (warp == 0) {
     const bool lead = elect_one();
@@ -1042,8 +1041,6 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
     const int pe = kEpiWarps == 8 ? (part ? kBN : kSplit) : kBN;
     const int total = a.sk_tiles * a.num_k;
     void* out = a.epi.out_slot ? *a.epi.out_slot : a.epi.out;
-    const bool h_ahead = FEAT == kFeatPlain && C::kStaging > 0 && a.epi.kind == SGD_EPI_DELTA;
-    float4 hv[8];  // first 32-column chunk of h (delta_staged)
     for (int u = 0; u < w.n_units; ++u) {
       int tile, k0, k1;
       unit_at(a, w, u, tile, k0, k1);
@@ -1055,13 +1052,12 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kBN;
       if (u >= w.n_sk) {  // data-parallel tile
         prefetch_h_row(a.epi, row, a.M, a.N, n_blk * kBN, cb, ce);
-        if (h_ahead) load_h_chunk(a, row - lane, n_blk * kBN + cb, hv);
         if (FEAT == kFeatH16 && a.epi.stat_cnt) {  // every epilogue thread reaches the barriers
           const bool ok = warp_wait(&tfull[acc], aph, abort_flag, a.status, 4);
           if (ok) {
             tc_fence_after();
             epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, cb, ce,
-                                                     part, kEpiWarps == 8 ? 2 : 1, stg, hv);
+                                                     part, kEpiWarps == 8 ? 2 : 1, stg);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -1072,7 +1068,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
         if (!warp_wait(&tfull[acc], aph, abort_flag, a.status, 4)) break;
         tc_fence_after();
         epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, cb, ce, part,
-                                           kEpiWarps == 8 ? 2 : 1, stg, hv);
+                                           kEpiWarps == 8 ? 2 : 1, stg);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -1083,10 +1079,9 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
       const bool ok = warp_wait(&tfull[acc], aph, abort_flag, a.status, 4);
       if (k0 == 0 && k1 == a.num_k) {  // the whole K range of the tile lies in this CTA's share
         if (ok) {
-          if (h_ahead) load_h_chunk(a, row - lane, n_blk * kBN + cb, hv);
-          tc_fence_after();
+            tc_fence_after();
           epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, cb, ce, part,
-                                           kEpiWarps == 8 ? 2 : 1, stg, hv);
+                                           kEpiWarps == 8 ? 2 : 1, stg);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -1123,7 +1118,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
       if (*last_flag != 0) {
         __threadfence();
         epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, WsSrc<kBN>{slot0, nseg, q * 32 + lane, a.epi.alpha},
-                                           cb, ce, part, kEpiWarps == 8 ? 2 : 1, stg, hv);
+                                           cb, ce, part, kEpiWarps == 8 ? 2 : 1, stg);
         if (threadIdx.x == 64) a.sk_cnt[tile] = 0;
       }
       // the CTA that finished the tile (last_flag is CTA-uniform) draws its row block's ticket

@@ -84,8 +84,8 @@ struct GemmPlan {
   int M = 0, N = 0, K = 0;   // N = output columns
   EpiParams epi{};
   bool simt = false;
-  bool allow_pair = false;   // let gemm_plan choose the CTA-pair kernel (gemm_pair_kernel.cuh)
-  bool pair = false;         // set by gemm_plan: the CTA-pair kernel, 256 x bn tiles
+  bool allow_group = false;  // let gemm_plan choose the CTA-group kernel (gemm_group_kernel.cuh)
+  int group = 0;             // set by gemm_plan: its CTAs per tile (2: 256 x bn, 1: 128 x bn), 0 the other kernel
   int bk = 64;               // K elements per stage: 64 (128-byte swizzle) or 32 (64-byte)
   int bn = 0;                // output columns per tile: 256, 128, or 0 = choose by tile count
   int epiw = 0;              // epilogue warps: 4, 8, or 0 = choose by epilogue kind
@@ -108,7 +108,6 @@ int gemm_plan(GemmPlan& p, const char** why);
 cudaError_t gemm_launch(const GemmPlan& p, cudaStream_t s);
 // fp32 elements of stream-K workspace a planned GEMM needs (0: data-parallel only).
 size_t gemm_ws_floats(const GemmPlan& p);
-int gemm_ws_tickets(const GemmPlan& p);  // and int tickets
 // The fixed stream-K scratch of the current device (partials, then tickets) and its
 // capacity; returns 0, or -1 with `why` set when its address cannot be obtained.
 size_t gemm_static_ws_bytes();

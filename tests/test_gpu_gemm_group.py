@@ -1,5 +1,5 @@
-"""The CTA-pair GEMM (sgd_kernel_gemm variant 0 where M > 128) against the oracle, at one shape
-per tile width and epilogue that the rule picks there, with ragged last tiles in M, N and K.
+"""The CTA-group GEMM (sgd_kernel_gemm variant 0) against the oracle, at one shape per group, tile
+width and epilogue that the rule picks there, with ragged last tiles in M, N and K.
 Bounds: fp16 results the rounding of the result plus fp32 accumulation; fp32 results
 accumulation alone, 2^-23 x sqrt(K) x the terms' norm with a factor of 8 for the tensor cores'
 truncation."""
@@ -25,17 +25,24 @@ def B():
     return binding
 
 
-# widths 128 (smallest, one column tile of 8, ragged), 160, 192, 224, 256
-SHAPES = [(129, 8, 8), (300, 520, 688), (2000, 1272, 328), (2048, 3456, 72), (2040, 3840, 136), (2048, 4600, 136),
-          (4000, 4096, 264), (4128, 4088, 512), (4128, 1016, 4096)]
+def _rows(rng, M):
+    """Up to 200 rows to compare: the first and last, a tile's edge, others at random."""
+    r = np.unique(np.r_[0, 127, 128, M - 1, rng.choice(M, min(M, 200), replace=False)])
+    return r[r < M]
+
+
+# one CTA of width 64 (one row and 8 columns; ragged; several waves), 128, 256; pairs of 160, 192,
+# 224, 256 and, with a long K, 128
+SHAPES = [(1, 8, 8), (128, 1000, 688), (257, 8200, 264), (333, 4096, 2056), (4012, 3024, 144), (1427, 1632, 464),
+          (3073, 824, 592), (1034, 2936, 872), (2852, 2696, 800), (333, 4096, 8200)]
 
 
 @pytest.mark.parametrize("M,N,K", SHAPES)
 @pytest.mark.parametrize("epi", ["f16", "f32", "gelu", "delta", "gate"])
-def test_pair_plain_and_residual(B, M, N, K, epi):
+def test_group_plain_and_residual(B, M, N, K, epi):
     rng = np.random.default_rng(M + N + K)
     A, W = _rand(rng, (M, K)).cuda(), _rand(rng, (N, K), 1 / math.sqrt(K)).cuda()
-    rows = np.unique(np.r_[0, 127, 128, M - 1, rng.choice(M, min(M, 200), replace=False)])
+    rows = _rows(rng, M)
     want = odn.linear(_f(A[rows]), _f(W))
     tol = 8 * 2.0 ** -23 * math.sqrt(K) + 1e-6  # of results of unit scale
     if epi in ("delta", "gate"):
@@ -62,14 +69,14 @@ def test_pair_plain_and_residual(B, M, N, K, epi):
     assert B.sgd_kernel_status() == 0
 
 
-@pytest.mark.parametrize("M,N,K", [(510, 8, 32), (2048, 1376, 136), (4096, 4600, 72)])
+@pytest.mark.parametrize("M,N,K", [(64, 688, 256), (383, 32, 8), (3217, 2624, 8), (272, 3592, 856), (1040, 3456, 784)])
 @pytest.mark.parametrize("act", [0, 1])
-def test_pair_gated(B, M, N, K, act):
+def test_group_gated(B, M, N, K, act):
     rng = np.random.default_rng(M + N + K + act)
     A, W = _rand(rng, (M, K)).cuda(), _rand(rng, (2 * N, K), 1 / math.sqrt(K)).cuda()
     out = torch.full((M, N), 7.0, dtype=torch.float16, device="cuda")
     B.sgd_kernel_gemm(A, W, M, N, K, B.sgd_epilogue_args(kind=B.EPI_GATED, out=out.data_ptr(), ldo=N, act=act))
-    rows = np.unique(np.r_[0, 127, 128, M - 1, rng.choice(M, 200, replace=False)])
+    rows = _rows(rng, M)
     u = odn.linear(_f(A[rows]), _f(W))
     want = u[:, :N] * odn.gelu_erf(u[:, N:]) if act else odn.silu(u[:, :N]) * u[:, N:]
     _check_f16(out[rows], want, extra_abs=2e-5 * float(np.abs(want).max()))
@@ -77,8 +84,8 @@ def test_pair_gated(B, M, N, K, act):
 
 
 @pytest.mark.parametrize("dh", [64, 128])
-@pytest.mark.parametrize("M,heads,K", [(129, 1, 16), (437, 5, 72), (2048, 8, 264)])
-def test_pair_rope(B, M, heads, K, dh):
+@pytest.mark.parametrize("M,heads,K", [(1, 1, 16), (100, 7, 72), (4146, 23, 16), (3382, 11, 776)])
+def test_group_rope(B, M, heads, K, dh):
     rng = np.random.default_rng(M + heads + K + dh)
     N, tokens, half = 3 * heads * dh, 50, dh // 2
     A, W = _rand(rng, (M, K)).cuda(), _rand(rng, (N, K), 1 / math.sqrt(K)).cuda()
