@@ -307,13 +307,6 @@ __device__ __forceinline__ bool warp_wait_bar(uint64_t* bar, uint32_t parity, vo
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-__device__ __forceinline__ void drain_bar(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = global_timer_ns();
-  while (!mbar_try_wait(bar, parity)) {
-    if (global_timer_ns() - t0 > kWaitTimeoutNs) break;
-  }
-}
-
 template <int DH>
 __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_constant__ AttnTcArgs a) {
   using L = TcLayout<DH>;
@@ -383,8 +376,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
         }
       }
       if (*abort_flag) {
-        drain_bar(q_full, 0);
-        for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) drain_bar(&kv_full[i & 1], (i >> 1) & 1);
+        mbar_drain(q_full, 0);
+        for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) mbar_drain(&kv_full[i & 1], (i >> 1) & 1);
       }
     }
   } else if (warp == 1) {
@@ -427,7 +420,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
         umma_commit(&o_done[s]);
       }
       umma_commit(drain);
-      drain_bar(drain, 0);
+      mbar_drain(drain, 0);
     }
   } else {
     const int q = warp & 3;
@@ -665,8 +658,8 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
       }
     }
     if (lead && *abort_flag) {
-      drain_bar(q_full, 0);
-      for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) drain_bar(&kv_full[i & 1], (i >> 1) & 1);
+      mbar_drain(q_full, 0);
+      for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) mbar_drain(&kv_full[i & 1], (i >> 1) & 1);
     }
   } else if (warp == 1) {
     // The whole warp runs the loop, one elected lane issues, and every operand of an MMA is a
@@ -736,7 +729,7 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
     }
     if (lead) {
       umma_commit(drain);
-      drain_bar(drain, 0);
+      mbar_drain(drain, 0);
     }
   } else {
     const int t = (warp - 2) >> 2;   // query tile of this warpgroup

@@ -251,6 +251,14 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
   }
 }
 
+// Bounded wait that ignores the abort flag (used while draining after an abort).
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+  const uint64_t t0 = global_timer_ns();
+  while (!mbar_try_wait(bar, parity)) {
+    if (global_timer_ns() - t0 > kWaitTimeoutNs) break;
+  }
+}
+
 // Whether the phase with parity `parity` has completed, without waiting (all lanes alike).
 __device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -305,6 +313,14 @@ __device__ __forceinline__ void tma_load_2d_at(uint32_t dst, const void* desc, u
       " [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(desc)), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
+}
+
+// Plain bulk copy of `bytes` (a multiple of 16; both addresses 16-byte aligned) into shared memory.
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(smem_dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
 }
 
 // ----------------------------------------------------------------------------

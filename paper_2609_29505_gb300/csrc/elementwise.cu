@@ -759,6 +759,105 @@ __global__ void __launch_bounds__(256) gemv_kernel(const GemvParams p) {
   }
 }
 
+// The same products for 2 to 8 rows and a large weight (the modulation of every active branch),
+// with the weight streamed through shared memory: an item's 32 columns are one contiguous block
+// of 64 K bytes, which a producer warp fetches whole (cp.async.bulk) into one of two buffers while
+// the other 8 warps multiply the item before it, 4 columns each.  With direct loads a warp had
+// only its own current columns in flight and stopped for every reduction: 56 x 3456 x 1152 took
+// 168 us for 446 MB.
+constexpr int kStreamCols = 32;
+constexpr int kStreamThreads = 288;
+inline size_t gemv_stream_smem(int K) {
+  return static_cast<size_t>(8) * K * sizeof(float) + 2 * static_cast<size_t>(kStreamCols) * K * sizeof(bf16) + 64;
+}
+
+__global__ void __launch_bounds__(kStreamThreads, 1) gemv_stream_kernel(const GemvParams p, int* status) {
+  extern __shared__ __align__(128) float xs[];  // x [8][2 planes][K / 2], two weight buffers, barriers
+  const int K = p.K, half = K >> 1;
+  uint8_t* wbuf = reinterpret_cast<uint8_t*>(xs + 8 * K);
+  const uint32_t wbytes = kStreamCols * K * sizeof(bf16);
+  uint64_t* full = reinterpret_cast<uint64_t*>(wbuf + 2 * wbytes);
+  uint64_t* empty = full + 2;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + 2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 8);
+    }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  pdl_wait_and_trigger();
+  const int k4 = K >> 2;
+  for (int i = threadIdx.x; i < 8 * k4; i += kStreamThreads) {
+    const int r = i / k4, k = (i - r * k4) << 2;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);  // rows past the last contribute nothing and are not stored
+    if (r < p.rows) x = __ldg(reinterpret_cast<const float4*>(p.x + static_cast<int64_t>(r) * p.ldx + k));
+    if (p.in_silu) x = make_float4(silu_f(x.x), silu_f(x.y), silu_f(x.z), silu_f(x.w));
+    *reinterpret_cast<float4*>(xs + r * K + ((k & 4) ? half : 0) + (k >> 3) * 4) = x;
+  }
+  __syncthreads();
+  const int per_seg = (p.N + kStreamCols - 1) / kStreamCols;
+  const int n_items = per_seg * (p.n_seg > 0 ? p.n_seg : 1);
+  if (warp == 8) {
+    if (lane == 0) {
+      int it = 0;
+      for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
+        const int s = it & 1;
+        if (!mbar_wait(&empty[s], ((it >> 1) & 1) ^ 1u, abort_flag, status, 41)) break;
+        const int seg = item / per_seg, j0 = (item - seg * per_seg) * kStreamCols;
+        const uint32_t bytes = min(kStreamCols, p.N - j0) * K * sizeof(bf16);  // K % 8 == 0: a multiple of 16
+        mbar_arrive_expect_tx(&full[s], bytes);
+        bulk_load(wbuf + s * wbytes, (p.n_seg ? p.w_seg[seg] : p.W) + static_cast<int64_t>(j0) * K, bytes, &full[s]);
+      }
+      if (*abort_flag)
+        for (int i = it > 2 ? it - 2 : 0; i < it; ++i) mbar_drain(&full[i & 1], (i >> 1) & 1);
+    }
+    return;
+  }
+  int it = 0;
+  for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
+    const int s = it & 1;
+    const int seg = item / per_seg, j0 = (item - seg * per_seg) * kStreamCols;
+    if (!mbar_wait_warp(smem_u32(&full[s]), (it >> 1) & 1, abort_flag, status, 42)) break;
+    const uint8_t* W = wbuf + s * wbytes + static_cast<size_t>(warp) * 4 * K * sizeof(bf16);
+    uint64_t acc2[32];  // [column][row], sums over even and odd k
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc2[i] = 0;
+    // (columns past N hold whatever the buffer held; their sums are not stored)
+    for (int k = lane * 8; k < K; k += 256) {
+      uint64_t wf[4][4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint4 w = *reinterpret_cast<const uint4*>(W + (static_cast<size_t>(c) * K + k) * sizeof(bf16));
+        const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) wf[c][q] = pack_f32x2(u[q] << 16, u[q] & 0xffff0000u);
+      }
+      const int xo = (k >> 3) * 4;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const ulonglong2 xa = *reinterpret_cast<const ulonglong2*>(xs + r * K + xo);
+        const ulonglong2 xb = *reinterpret_cast<const ulonglong2*>(xs + r * K + half + xo);
+        const uint64_t xv[4] = {xa.x, xa.y, xb.x, xb.y};
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) fma_f32x2(acc2[c * 8 + r], wf[c][q], xv[q]);
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+    float acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = sum_f32x2(acc2[i]);
+    const float v = transpose_reduce32(acc, lane);
+    const int j = j0 + warp * 4 + lane / 8, r = lane % 8;
+    if (r < p.rows && j < p.N) gemv_store(p, p.n_seg ? p.out_seg[seg] : p.out, r, j, v);
+  }
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1053,6 +1152,15 @@ cudaError_t gemv_launch(const GemvParams& p, cudaStream_t s) {
   if (xrows == 1) {
     const bool few = static_cast<int64_t>(p.N) * std::max(p.n_seg, 1) < 64ll * num_sms();
     return few ? gemv_launch_r<1, 1>(p, smem, s) : gemv_launch_r<1, 4>(p, smem, s);
+  }
+  // many columns of a wide-enough weight to keep every SM streaming, and buffers that fit
+  const int64_t items = static_cast<int64_t>((p.N + kStreamCols - 1) / kStreamCols) * std::max(p.n_seg, 1);
+  if (xrows <= 8 && items >= 2 * num_sms() && gemv_stream_smem(p.K) <= 220 * 1024) {
+    const size_t bytes = gemv_stream_smem(p.K);
+    cudaError_t e = cudaFuncSetAttribute(gemv_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(bytes));
+    if (e != cudaSuccess) return e;
+    return launch_k(gemv_stream_kernel, dim3(num_sms()), dim3(kStreamThreads), bytes, s, p, device_status_ptr());
   }
   if (xrows <= 8) return gemv_launch_r<8, 4>(p, smem, s);
   return gemv_launch_r<16, 2>(p, smem, s);

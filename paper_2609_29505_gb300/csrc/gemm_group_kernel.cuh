@@ -293,10 +293,10 @@ __device__ __forceinline__ void gemm_group_body(const TcArgs& a) {
     if (*abort_flag) {
       // both CTAs' loads still in flight; the other CTA stays at the cluster barrier meanwhile
       if (lead && rank == 0)
-        for (int i = tail; i < it; ++i) drain_wait(&full[i % kStages], (i / kStages) & 1);
+        for (int i = tail; i < it; ++i) mbar_drain(&full[i % kStages], (i / kStages) & 1);
     } else if (lead) {
       // the releases committed to this CTA's barriers arrive before it ends
-      for (int i = tail; i < it; ++i) drain_wait(&empty[i % kStages], (i / kStages) & 1);
+      for (int i = tail; i < it; ++i) mbar_drain(&empty[i % kStages], (i / kStages) & 1);
     }
   } else if (warp == 1) {
     if (rank == 0) {
@@ -348,7 +348,7 @@ __device__ __forceinline__ void gemm_group_body(const TcArgs& a) {
       if (lead) umma_commit_group<CG>(smem_u32(drain));
     }
     // every MMA has finished, and the leader has committed for the last time, once `drain` completes
-    if (lane == 0) drain_wait(drain, 0);
+    if (lane == 0) mbar_drain(drain, 0);
   } else {
     float4* stg = reinterpret_cast<float4*>(tiles + kStages * kStageBytes + 512) + (warp - 2) * 256;
     const int q = warp & 3, part = (warp - 2) >> 2;

@@ -735,14 +735,6 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
   return ok != 0;
 }
 
-// Bounded wait that ignores the abort flag (used while draining after an abort).
-__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = global_timer_ns();
-  while (!mbar_try_wait(bar, parity)) {
-    if (global_timer_ns() - t0 > kWaitTimeoutNs) break;
-  }
-}
-
 // Named barrier 1 over the epilogue warps, returning the AND of `v` over them.
 __device__ __forceinline__ bool epi_bar_and(bool v, int nthreads) {
   uint32_t r;
@@ -961,7 +953,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
     if (lead && *abort_flag) {
       // wait for the loads still in flight (the latest issue of each stage)
       for (int i = (it > kStages ? it - kStages : 0); i < it; ++i)
-        drain_wait(&full[i % kStages], (i / kStages) & 1);
+        mbar_drain(&full[i % kStages], (i / kStages) & 1);
     }
   } else if (warp == 1) {
     // The whole warp runs the loop and one elected lane issues.  A K-block is 256 (BN 128) to
@@ -1023,7 +1015,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
     if (lead) {
       // every MMA issued by this thread has finished once `drain` completes
       umma_commit(drain);
-      drain_wait(drain, 0);
+      mbar_drain(drain, 0);
     }
   } else {
     const int q = warp & 3;
