@@ -3,9 +3,11 @@
 // Used inside every active self-attention and cross-attention branch (Algorithm 2:
 // an active unit evaluates F_l(h_{l-1,s}; c_s)); frozen units never launch it.
 //
-// Three kernels:
-//   attn_pp_kernel (d_h 64, 128; the default): tcgen05 with two query tiles per CTA and two
-//     alternating softmax warpgroups, P in TMEM; described above the kernel.
+// Four kernels:
+//   attn_pp_kernel (d_h 64, 72, 128; long or many sequences): tcgen05 with two query tiles per
+//     CTA and two alternating softmax warpgroups, P in TMEM; described above the kernel.
+//   attn_sm_kernel (d_h 64, 72, 128; few keys or an ill-fitting last wave, by attn_small): tcgen05
+//     with one query tile per CTA, key tiles of 64, and several CTAs per SM.
 //   attn_tc_kernel (d_h 64, 128): tcgen05.  One CTA = 128 queries of one (sample, head),
 //     keys in tiles of 128.  Warp 0 loads Q once and K/V tiles through a 2-stage TMA ring;
 //     warp 1 issues S = Q K^T into one of two TMEM S buffers and O += P V into a TMEM O
@@ -22,6 +24,8 @@
 // registers (exp2 with the scale folded in).  Q, K, V, P and O are fp16 (m16n8k16
 // f16 x f16 -> f32).  Keys beyond n_kv are masked and their
 // shared-memory rows zero-filled; head dims 72 are padded to 80 in shared memory.
+#include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "common.cuh"
@@ -837,18 +841,271 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
   }
 }
 
+// ----------------------------------------------------------------------------
+// attn_sm_kernel: one query tile per CTA, key tiles of 64, several CTAs per SM.
+//
+// A CTA of attn_pp_kernel holds an SM alone, so that with few key tiles its prologue, first
+// loads, the chain of its tiles and the last stores are all exposed, and a second wave of a few
+// CTAs costs a whole one.  Here one CTA = 128 queries with S (64 fp32 columns) and O in 128 (d_h
+// 64) or 256 columns of TMEM and 50 to 100 KB of shared memory: 3 (d_h 64) or 2 CTAs share an SM
+// and cover each other's latencies, ragged key counts waste at most 63 keys, and a warp whose 32
+// queries do not exist skips its softmax.  P overwrites S as in attn_pp_kernel.
+// ----------------------------------------------------------------------------
+constexpr int kSmThreads = 192;
+constexpr int kSmBK = 64;
+
 template <int DH>
-cudaError_t launch_pp(const AttnPlan& plan, cudaStream_t s) {
-  using L = PpLayout<DH>;
-  static bool done[64] = {false};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(attn_pp_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         L::kBytes);
-    if (e != cudaSuccess) return e;
-    done[dev] = true;
+struct SmLayout {
+  static constexpr bool kPad = DH == 72;
+  static constexpr int kA64 = DH / 64, kA16 = kPad ? 1 : 0;
+  static constexpr int kDP = 64 * kA64 + 16 * kA16;   // head width the MMAs see
+  static constexpr int kAtomKV = kSmBK * 128, kAtomKV32 = kSmBK * 32;
+  static constexpr int kQBytes = kA64 * kAtom + kA16 * kAtom32;
+  static constexpr int kTile = kA64 * kAtomKV + kA16 * kAtomKV32;
+  static constexpr int kStage = 2 * kTile;            // the K tile, then the V tile
+  static constexpr int kKV = kQBytes;
+  static constexpr int kBar = kKV + 2 * kStage;
+  static constexpr int kBytes = kBar + 128 + 1024;
+  static constexpr int kTmemCols = kSmBK + kDP <= 128 ? 128 : 256;
+  static constexpr int kBlocks = DH == 64 ? 3 : 2;    // per SM
+  static constexpr uint32_t kTmemO = kSmBK;
+  static_assert(kKV % 1024 == 0 && kTile % 1024 == 0 && kStage % 1024 == 0, "swizzle atoms");
+  static_assert(kBlocks * (kBytes + 1024) <= 233472 && kBlocks * kTmemCols <= 512, "CTAs per SM");
+};
+
+template <int DH>
+__global__ void __launch_bounds__(kSmThreads, SmLayout<DH>::kBlocks) attn_sm_kernel(const __grid_constant__ AttnTcArgs a) {
+  using L = SmLayout<DH>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kBar);
+  uint64_t* q_full = bars;
+  uint64_t* kv_full = bars + 1;
+  uint64_t* kv_empty = bars + 3;
+  uint64_t* s_full = bars + 5;
+  uint64_t* p_full = bars + 6;
+  uint64_t* o_done = bars + 7;
+  uint64_t* drain = bars + 8;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 9);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int qt = blockIdx.x, bh = blockIdx.y;
+  const int b = bh / a.n_heads, h = bh % a.n_heads;
+  const int nt = (a.n_kv + kSmBK - 1) / kSmBK;
+
+  if (threadIdx.x == 0) {
+    tma_prefetch_desc(&a.tmap_q);
+    tma_prefetch_desc(&a.tmap_k);
+    tma_prefetch_desc(&a.tmap_v);
+    mbar_init(q_full, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&kv_full[i], 1);
+      mbar_init(&kv_empty[i], 1);
+    }
+    mbar_init(s_full, 1);
+    mbar_init(p_full, 4);
+    mbar_init(o_done, 1);
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
   }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, L::kTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_wait_and_trigger();  // the prologue above touched only shared memory and TMEM
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    const bool lead = elect_one();
+    const uint32_t sm0 = smem_u32(sm), kv_full0 = smem_u32(kv_full), kv_empty0 = smem_u32(kv_empty);
+    const int col0 = h * a.head_stride;
+    if (lead) {
+      const uint32_t bar = smem_u32(q_full);
+      const int row = b * a.n_q + qt * kTcBQ;
+      mbar_arrive_expect_tx_at(bar, L::kQBytes);
+      for (int at = 0; at < L::kA64; ++at) tma_load_2d_at(sm0 + at * kAtom, &a.tmap_q, bar, col0 + at * 64, row);
+      if (L::kPad) tma_load_2d_at(sm0 + L::kA64 * kAtom, &a.tmap_q16, bar, col0 + 64, row);
+    }
+    int j = 0;
+    for (; j < nt; ++j) {
+      const int s = j & 1;
+      if (!mbar_wait_warp(kv_empty0 + 8 * s, ((j >> 1) & 1) ^ 1u, abort_flag, a.status, 51)) break;
+      if (lead) {
+        const uint32_t st = sm0 + L::kKV + s * L::kStage, bar = kv_full0 + 8 * s;
+        const int row = b * a.n_kv + j * kSmBK;
+        mbar_arrive_expect_tx_at(bar, 2 * L::kTile);
+        for (int at = 0; at < L::kA64; ++at) tma_load_2d_at(st + at * L::kAtomKV, &a.tmap_k, bar, col0 + at * 64, row);
+        if (L::kPad) tma_load_2d_at(st + L::kA64 * L::kAtomKV, &a.tmap_k16, bar, col0 + 64, row);
+        for (int at = 0; at < L::kA64; ++at)
+          tma_load_2d_at(st + L::kTile + at * L::kAtomKV, &a.tmap_v, bar, col0 + at * 64, row);
+        if (L::kPad) tma_load_2d_at(st + L::kTile + L::kA64 * L::kAtomKV, &a.tmap_v16, bar, col0 + 64, row);
+      }
+    }
+    if (lead && *abort_flag) {
+      mbar_drain(q_full, 0);
+      for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) mbar_drain(&kv_full[i & 1], (i >> 1) & 1);
+    }
+  } else if (warp == 1) {
+    const bool lead = elect_one();
+    constexpr uint32_t idesc_qk = umma_idesc_f16(kTcBQ, kSmBK);
+    constexpr uint32_t idesc_pv = umma_idesc_f16_bmn(kTcBQ, 64 * L::kA64);
+    constexpr uint32_t idesc_pv16 = umma_idesc_f16_bmn(kTcBQ, 16);
+    const uint32_t sm0 = smem_u32(sm), kv_full0 = smem_u32(kv_full), kv_empty0 = smem_u32(kv_empty);
+    const uint64_t dq = smem_desc_sw128(sm0), dk = smem_desc_sw128(sm0 + L::kKV);
+    const uint64_t dv = smem_desc_sw128_mn(sm0 + L::kKV + L::kTile, L::kAtomKV, 1024);
+    const uint64_t dq16 = smem_desc_sw32(sm0 + L::kA64 * kAtom);
+    const uint64_t dk16 = smem_desc_sw32(sm0 + L::kKV + L::kA64 * L::kAtomKV);
+    const uint64_t dv16 = smem_desc_sw32_mn(sm0 + L::kKV + L::kTile + L::kA64 * L::kAtomKV, L::kAtomKV32, 256);
+    constexpr uint64_t kStageU = L::kStage >> 4;
+    auto issue_qk = [&](int s) {
+      if (!lead) return;
+      const uint64_t ka = dk + s * kStageU;
+#pragma unroll
+      for (int ks = 0; ks < 4 * L::kA64; ++ks)
+        umma_f16(tmem, dq + (((ks >> 2) * kAtom + (ks & 3) * 32) >> 4),
+                 ka + (((ks >> 2) * L::kAtomKV + (ks & 3) * 32) >> 4), idesc_qk, ks > 0 ? 1u : 0u);
+      if (L::kPad) umma_f16(tmem, dq16, dk16 + s * kStageU, idesc_qk, 1u);  // head columns 64..79
+      umma_commit_at(smem_u32(s_full));
+    };
+    bool ok = mbar_wait_warp(smem_u32(q_full), 0, abort_flag, a.status, 52) &&
+              mbar_wait_warp(kv_full0, 0, abort_flag, a.status, 53);
+    if (ok) {
+      tc_fence_after();
+      issue_qk(0);
+    }
+    for (int j = 0; j < nt && ok; ++j) {
+      const int s = j & 1;
+      if (!(ok = mbar_wait_warp(smem_u32(p_full), j & 1, abort_flag, a.status, 54))) break;
+      tc_fence_after();
+      if (lead) {
+        const uint64_t va = dv + s * kStageU, va16 = dv16 + s * kStageU;
+        const uint32_t acc = j > 0 ? 1u : 0u;
+#pragma unroll
+        for (int ks = 0; ks < kSmBK / 16; ++ks) {
+          umma_f16_ts(tmem + L::kTmemO, tmem + 8 * ks, va + ks * (2048 >> 4), idesc_pv, ks > 0 ? 1u : acc);
+          if (L::kPad)  // O columns 64..79
+            umma_f16_ts(tmem + L::kTmemO + 64 * L::kA64, tmem + 8 * ks, va16 + ks * (512 >> 4), idesc_pv16,
+                        ks > 0 ? 1u : acc);
+        }
+        umma_commit_at(kv_empty0 + 8 * s);
+        umma_commit_at(smem_u32(o_done));
+      }
+      if (j + 1 < nt) {
+        if (!(ok = mbar_wait_warp(kv_full0 + 8 * (s ^ 1), ((j + 1) >> 1) & 1, abort_flag, a.status, 55))) break;
+        tc_fence_after();
+        issue_qk(s ^ 1);  // after PV(j) in issue order, which reads P where S goes
+      }
+    }
+    if (lead) {
+      umma_commit(drain);
+      mbar_drain(drain, 0);
+    }
+  } else {
+    const int q = warp & 3;
+    const int row = q * 32 + lane, qrow = qt * kTcBQ + row;
+    const uint32_t s_col = tmem + (static_cast<uint32_t>(q * 32) << 16), o_col = s_col + L::kTmemO;
+    const bool any = qt * kTcBQ + q * 32 < a.n_q;  // warp-uniform: some of its queries exist
+    float m2 = -INFINITY, l = 0.f;
+    bool ok = true;
+    uint32_t r[kSmBK];
+    for (int j = 0; j < nt && ok; ++j) {
+      if (!(ok = mbar_wait_warp(smem_u32(s_full), j & 1, abort_flag, a.status, 56))) break;
+      tc_fence_after();
+      if (any) {
+        const int nvalid = min(a.n_kv - j * kSmBK, kSmBK);  // keys of this tile (the rest are masked)
+#pragma unroll
+        for (int c = 0; c < kSmBK; c += 16) tmem_ld16(s_col + c, r + c);
+#pragma unroll
+        for (int c = 0; c < kSmBK; c += 16) tmem_ld_wait16(r + c);
+        if (nvalid < kSmBK) {
+#pragma unroll
+          for (int c = 0; c < kSmBK; ++c)
+            if (c >= nvalid) r[c] = __float_as_uint(-INFINITY);
+        }
+        float mx[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) mx[i] = __uint_as_float(r[i]);
+#pragma unroll
+        for (int c = 4; c < kSmBK; ++c) mx[c & 3] = fmaxf(mx[c & 3], __uint_as_float(r[c]));
+        const float mt = a.scale_log2 * fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        if (j == 0) {
+          m2 = mt;
+        } else if (__any_sync(0xffffffffu, mt > m2 + kRescaleLog2)) {
+          // warp-uniform (the TMEM accesses are .sync.aligned); O must hold PV(j-1)
+          if (!(ok = mbar_wait_warp(smem_u32(o_done), (j - 1) & 1, abort_flag, a.status, 57))) break;
+          tc_fence_after();
+          const float mnew = fmaxf(m2, mt);
+          const float corr = exp2f(m2 - mnew);
+          uint32_t o16[16];
+#pragma unroll 1
+          for (int c = 0; c < L::kDP; c += 16) {
+            tmem_ld16(o_col + c, o16);
+            tmem_ld_wait16(o16);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) o16[i] = __float_as_uint(__uint_as_float(o16[i]) * corr);
+            tmem_st16(o_col + c, o16);
+          }
+          tmem_st_wait();
+          l *= corr;
+          m2 = mnew;
+        }
+        const float neg_m2 = -m2;
+        float ls[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ls[i] = 0.f;
+#pragma unroll
+        for (int c = 0; c < kSmBK; c += 32) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const float p0 = ex2_approx(fmaf(__uint_as_float(r[c + 2 * k]), a.scale_log2, neg_m2));
+            const float p1 = ex2_approx(fmaf(__uint_as_float(r[c + 2 * k + 1]), a.scale_log2, neg_m2));
+            ls[k & 3] += p0 + p1;
+            r[c + k] = pack_f16x2_rn(p0, p1);
+          }
+          tmem_st16(s_col + c / 2, r + c);
+        }
+        l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        tmem_st_wait();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full);
+    }
+    if (ok && mbar_wait_warp(smem_u32(o_done), (nt - 1) & 1, abort_flag, a.status, 58) && any) {
+      tc_fence_after();
+      const float inv = 1.f / l;
+      f16* orow = a.o + (static_cast<int64_t>(b) * a.n_q + qrow) * a.ldo + h * DH;
+#pragma unroll
+      for (int c = 0; c < L::kDP; c += 16) {
+        tmem_ld16(o_col + c, r);
+        tmem_ld_wait16(r);
+        float f[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(r[i]) * inv;
+        if (qrow < a.n_q) {
+          reinterpret_cast<uint4*>(orow + c)[0] = pack_f16x8(f);
+          if (c + 16 <= DH) reinterpret_cast<uint4*>(orow + c)[1] = pack_f16x8(f + 8);
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) {
+    __syncwarp();
+    tmem_dealloc(tmem, L::kTmemCols);
+  }
+}
+
+template <int DH>
+AttnTcArgs tc_args(const AttnPlan& plan) {
   const AttnParams& p = plan.p;
   AttnTcArgs a;
   memcpy(&a.tmap_q, &plan.tmap_q, sizeof(CUtensorMap));
@@ -865,8 +1122,40 @@ cudaError_t launch_pp(const AttnPlan& plan, cudaStream_t s) {
   a.n_heads = p.n_heads;
   a.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(DH));
   a.status = device_status_ptr();
+  return a;
+}
+
+template <int DH>
+cudaError_t launch_sm(const AttnPlan& plan, cudaStream_t s) {
+  using L = SmLayout<DH>;
+  static bool done[64] = {false};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(attn_sm_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         L::kBytes);
+    if (e != cudaSuccess) return e;
+    done[dev] = true;
+  }
+  dim3 grid((plan.p.n_q + kTcBQ - 1) / kTcBQ, plan.p.batch * plan.p.n_heads);
+  return launch_k(attn_sm_kernel<DH>, grid, dim3(kSmThreads), L::kBytes, s, tc_args<DH>(plan));
+}
+
+template <int DH>
+cudaError_t launch_pp(const AttnPlan& plan, cudaStream_t s) {
+  using L = PpLayout<DH>;
+  static bool done[64] = {false};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(attn_pp_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         L::kBytes);
+    if (e != cudaSuccess) return e;
+    done[dev] = true;
+  }
+  const AttnParams& p = plan.p;
   dim3 grid((p.n_q + kPpBQ - 1) / kPpBQ, p.batch * p.n_heads);
-  return launch_k(attn_pp_kernel<DH>, grid, dim3(kPpThreads), L::kBytes, s, a);
+  return launch_k(attn_pp_kernel<DH>, grid, dim3(kPpThreads), L::kBytes, s, tc_args<DH>(plan));
 }
 
 template <int DH>
@@ -949,6 +1238,26 @@ int attn_check(const AttnParams& p, const char** why) {
   return 0;
 }
 
+// Whether attn_sm_kernel runs this shape faster than attn_pp_kernel, by the time of each in us:
+// a pair CTA holds an SM for a fixed part and ~1.2 us per 128 keys; a CTA of attn_sm_kernel takes
+// ~1 us per 64 keys by itself, and the SM ~0.5 us (d_h 64; 0.6, 0.8) for one of several.  Fitted to
+// 22 shapes (measured us, pair / this kernel):
+//   16 x 258 tokens, 16 heads of 64    27.0 / 17.3     2 x 1024, 20 heads of 64         26.4 / 22.1
+//   2 x 1024 x 77 keys, 20 heads of 64 10.9 /  7.0     4 x 512, 16 heads of 64           9.4 / 11.3
+//   1 x 333, 32 heads of 128           10.3 /  9.9     4 x 1024, 32 heads of 128        76.6 / 90.3
+//   8 x 256, 16 heads of 72             8.3 /  8.8     2 x 136, 16 heads of 72           7.8 /  6.4
+bool attn_small(const AttnParams& p) {
+  const double sms = num_sms(), heads = static_cast<double>(p.batch) * p.n_heads;
+  const double pairs = std::ceil(p.n_q / 256.0) * heads, ctas = std::ceil(p.n_q / 128.0) * heads;
+  const double nt = std::ceil(p.n_kv / 128.0), nt64 = std::ceil(p.n_kv / 64.0);
+  const bool d64 = p.d_head == 64, d72 = p.d_head == 72;
+  const double pair_fixed = p.d_head == 128 ? 5.0 : 3.0, pair_tile = d64 ? 1.14 : (d72 ? 1.3 : 1.15);
+  const double sm_tile = d64 ? 0.52 : (d72 ? 0.6 : 0.8), slots = sms * (d64 ? 3 : 2);
+  const double t_pair = std::ceil(pairs / sms) * (pair_fixed + nt * pair_tile);
+  const double t_small = 2.0 + nt64 * std::max(std::ceil(ctas / slots), sm_tile * ctas / sms);
+  return t_small < t_pair;
+}
+
 int attn_plan(AttnPlan& plan, const char** why) {
   const AttnParams& p = plan.p;
   int rc = attn_check(p, why);
@@ -960,19 +1269,19 @@ int attn_plan(AttnPlan& plan, const char** why) {
   const bool tc_dh = p.d_head == 64 || p.d_head == 128 || (pad72 && p.impl != 2);
   plan.tc = (p.impl == 0 || p.impl == 2 || p.impl == 3) && tc_dh;
   if (!plan.tc) return 0;
-  // two query tiles per CTA (ping-pong) unless one tile per CTA is forced: faster on every
-  // measured shape, short and ragged ones included (258 tokens: 37.8 against 55.2 us)
   plan.pp = p.impl == 0 || p.impl == 3;
+  plan.small = p.impl == 0 && attn_small(p);
+  const int bk = plan.small ? kSmBK : kTcBK;
   const int cols = (p.n_heads - 1) * hs + (pad72 ? 80 : p.d_head);
   if (!make_tmap_f16(&plan.tmap_q, p.q, p.batch * p.n_q, cols, p.ldq, kTcBQ) ||
-      !make_tmap_f16(&plan.tmap_kv, p.k, p.batch * p.n_kv, cols, p.ldkv, kTcBK) ||
-      !make_tmap_f16(&plan.tmap_v, p.v, p.batch * p.n_kv, cols, p.ldkv, kTcBK)) {
+      !make_tmap_f16(&plan.tmap_kv, p.k, p.batch * p.n_kv, cols, p.ldkv, bk) ||
+      !make_tmap_f16(&plan.tmap_v, p.v, p.batch * p.n_kv, cols, p.ldkv, bk)) {
     *why = "attention: cuTensorMapEncodeTiled failed";
     return -5;
   }
   if (pad72 && (!make_tmap_f16(&plan.tmap_q16, p.q, p.batch * p.n_q, cols, p.ldq, kTcBQ, 16) ||
-                !make_tmap_f16(&plan.tmap_k16, p.k, p.batch * p.n_kv, cols, p.ldkv, kTcBK, 16) ||
-                !make_tmap_f16(&plan.tmap_v16, p.v, p.batch * p.n_kv, cols, p.ldkv, kTcBK, 16))) {
+                !make_tmap_f16(&plan.tmap_k16, p.k, p.batch * p.n_kv, cols, p.ldkv, bk, 16) ||
+                !make_tmap_f16(&plan.tmap_v16, p.v, p.batch * p.n_kv, cols, p.ldkv, bk, 16))) {
     *why = "attention: cuTensorMapEncodeTiled failed";
     return -5;
   }
@@ -981,6 +1290,8 @@ int attn_plan(AttnPlan& plan, const char** why) {
 
 cudaError_t attn_launch(const AttnPlan& plan, cudaStream_t s) {
   const AttnParams& p = plan.p;
+  if (plan.tc && plan.small)
+    return p.d_head == 64 ? launch_sm<64>(plan, s) : (p.d_head == 72 ? launch_sm<72>(plan, s) : launch_sm<128>(plan, s));
   if (plan.tc && plan.pp)
     return p.d_head == 64 ? launch_pp<64>(plan, s) : (p.d_head == 72 ? launch_pp<72>(plan, s) : launch_pp<128>(plan, s));
   if (plan.tc) return p.d_head == 64 ? launch_tc<64>(plan, s) : launch_tc<128>(plan, s);

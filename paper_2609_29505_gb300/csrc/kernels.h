@@ -131,9 +131,9 @@ struct AttnParams {
   f16* o;
   int ldo;
   int batch, n_q, n_kv, n_heads, d_head;
-  int impl;  // 0: tcgen05 with two query tiles per CTA where d_head is 64 or 128 (72 from a
-             //    head-padded layout), else mma.sync; 1: mma.sync; 2: tcgen05, one query
-             //    tile per CTA; 3: same as 0
+  int impl;  // 0: tcgen05 where d_head is 64 or 128 (72 from a head-padded layout), with one or
+             //    two query tiles per CTA by shape, else mma.sync; 1: mma.sync; 2: tcgen05, one
+             //    query tile per CTA, P in shared memory; 3: tcgen05, two query tiles per CTA
   int head_stride;  // input (q, k, v) columns between heads; 0 = d_head.  Outputs: d_head.
 };
 // A planned attention launch: parameters plus TMA descriptors for the tcgen05 kernel.
@@ -141,6 +141,7 @@ struct AttnPlan {
   AttnParams p{};
   bool tc = false;
   bool pp = false;  // two query tiles per CTA (attn_pp_kernel)
+  bool small = false;  // one query tile per CTA, several CTAs per SM (attn_sm_kernel)
   CUtensorMap tmap_q;
   CUtensorMap tmap_kv;
   CUtensorMap tmap_v;
