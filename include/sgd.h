@@ -102,9 +102,9 @@ typedef enum {
 /* Use 64-element K-blocks (4 stages, 128-byte swizzle) in the tcgen05 GEMMs. */
 #define SGD_FLAG_GEMM_BK64 8
 /* Launch a step's kernels with programmatic dependent launch: each kernel's launch and
- * prologue overlap the previous kernel's tail (by default a kernel starts only after the
- * previous one has finished).  Measured on GB300 it gains nothing on the mid-size models
- * and loses 1.5% on the LLaDA-8B-shaped step, whose clock falls under the power cap. */
+ * prologue overlap the previous kernel's tail.  Every context does so (measured on GB300: tiny
+ * -7%, DiT, U-ViT and SDXL-shaped -2 to -3%, LLaDA-8B-shaped -1% of the step's time; results are
+ * the same bit for bit), so the flag is accepted and changes nothing. */
 #define SGD_FLAG_PDL 16
 /* Fold RMSNorm / LayerNorm pre-norms into the GEMMs that follow them (Algorithm 2's
  * Norm -> projection as one tcgen05 GEMM: the gain folded into the weight, the row

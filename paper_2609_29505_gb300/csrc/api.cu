@@ -155,7 +155,7 @@ struct sgd_ctx {
   int M = 0, U = 0, nbr = 0;
   int attn_impl = 0;  // 1: mma.sync attention everywhere (SGD_FLAG_MMA_SYNC_ATTENTION)
   int head_stride = 0;  // columns per head in qkv: d_head, or 80 for d_head 72 on tcgen05
-  bool pdl = false;     // programmatic dependent launch between a step program's kernels
+  bool pdl = true;      // programmatic dependent launch between a step program's kernels
   int gemm_bk = 64;   // default K-block of the tcgen05 GEMM
   int exec_mode = SGD_EXEC_JAGGED_GRAPH;
   float* h_pad = nullptr;  // padded mode: residual that discarded branch updates land in
@@ -1193,7 +1193,11 @@ int sgd_create(const sgd_model_desc* desc, const sgd_weights* w, sgd_ctx** out) 
   }
   c->M = desc->batch * desc->n_tokens;
   c->attn_impl = (desc->flags & SGD_FLAG_MMA_SYNC_ATTENTION) ? 1 : 0;
-  c->pdl = (desc->flags & SGD_FLAG_PDL) != 0;
+  // A step is 20 to 200 kernels of 4 to 30 us (mid-size models), and the gap between two of them
+  // was ~2 us: with each kernel's launch and prologue inside its predecessor's tail the steps of
+  // the tiny / DiT / U-ViT / SDXL-shaped models take 672 / 5815 / 1627 / 617 us instead of 724 / 6000 /
+  // 1655 / 638 (whole short trajectories), the LLaDA-shaped blocks 8350 instead of 8430.
+  c->pdl = true;
   // RMSNorm / LayerNorm pre-norms fold into the GEMMs that follow them on request; the AdaLN
   // modulation (a per-sample scale of the weight's columns) and the SIMT debug GEMM do not
   c->fold = (desc->norm == SGD_NORM_RMS || desc->norm == SGD_NORM_LN) &&
