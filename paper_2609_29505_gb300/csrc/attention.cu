@@ -266,14 +266,6 @@ __device__ __forceinline__ uint32_t pack_f16x2_rn(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// 2^x with the hardware's approximate base-2 exponential (PTX ex2.approx.ftz.f32); the
-// arguments here are <= 8 and results below the fp16 range flush to zero either way.
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 struct AttnTcArgs {
   CUtensorMap tmap_q;
   CUtensorMap tmap_k;

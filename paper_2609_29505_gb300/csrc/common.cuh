@@ -130,6 +130,33 @@ __device__ __forceinline__ float gelu_tanh_f(float x) {
   return __fdividef(x, 1.0f + __expf(-c2 * (x + 0.044715f * x * x * x)));
 }
 
+// 2^x with the hardware's approximate base-2 exponential (PTX ex2.approx.ftz.f32).
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// x0 / (1 + 2^t0) and x1 / (1 + 2^t1) with one reciprocal, r = 1 / (d0 d1): the special-function unit
+// (an exponential and a reciprocal per value) bounded the GELU and SwiGLU epilogues.  Above
+// t = 62 the factor is taken as 0 (it is under 2^-62; x times it is x / inf in the limit, NaN for an
+// infinite x), and the exponents are held there so that d0 d1 stays in range.
+__device__ __forceinline__ void sigmoid_scale2(float& x0, float& x1, float t0, float t1) {
+  const float d0 = 1.0f + ex2_approx(fminf(t0, 62.f)), d1 = 1.0f + ex2_approx(fminf(t1, 62.f));
+  const float r = __fdividef(1.0f, d0 * d1);
+  x0 *= t0 > 62.f ? 0.f : r * d1;
+  x1 *= t1 > 62.f ? 0.f : r * d0;
+}
+__device__ __forceinline__ void silu2(float& x0, float& x1) {
+  constexpr float k = -1.4426950408889634f;  // -log2(e)
+  sigmoid_scale2(x0, x1, k * x0, k * x1);
+}
+__device__ __forceinline__ void gelu_tanh2(float& x0, float& x1) {
+  constexpr float k0 = -2.0f * 0.79788456080286536f * 1.4426950408889634f;  // -2 sqrt(2/pi) log2(e)
+  constexpr float k1 = 0.044715f * k0;
+  sigmoid_scale2(x0, x1, x0 * fmaf(k1, x0 * x0, k0), x1 * fmaf(k1, x1 * x1, k0));
+}
+
 // ----------------------------------------------------------------------------
 // shared-memory addresses, timers
 // ----------------------------------------------------------------------------

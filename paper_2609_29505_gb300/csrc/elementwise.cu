@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(128) stem_rows_kernel(const StemParams p) {
 // patches it has put in shared memory (read by every thread alike).  One thread per (row, 4
 // channels) read its 4 weight rows again for every row, 32 different lines per load: 22 us for
 // 2048 x 1152.  Each channel's dot product is summed in k order as in stem_kernel.
-constexpr int kPatchRows = 16;
+constexpr int kPatchRows = 8;
 template <int DIN>
 __global__ void __launch_bounds__(128) stem_patch_kernel(const StemParams p) {
   __shared__ float4 zs[kPatchRows][DIN / 4];
@@ -533,9 +533,12 @@ __global__ void __launch_bounds__(128) stem_patch_kernel(const StemParams p) {
   }
   __syncthreads();
   if (!active) return;
+  uint2 pos_next = __ldg(reinterpret_cast<const uint2*>(p.pos + static_cast<int64_t>(r0 % p.n_tokens) * p.d + c0));
 #pragma unroll 1
   for (int k = 0; k < nr; ++k) {
     const int r = r0 + k, n = r % p.n_tokens, b = r / p.n_tokens;
+    const float4 ps = bf16x4(pos_next);
+    pos_next = __ldg(reinterpret_cast<const uint2*>(p.pos + static_cast<int64_t>((r + 1) % p.n_tokens) * p.d + c0));
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (n < p.n_prefix) {
       const int cls = min(max(s->class_ids[b], 0), p.n_classes - 1);
@@ -551,7 +554,6 @@ __global__ void __launch_bounds__(128) stem_patch_kernel(const StemParams p) {
         v.w = fmaf(z.w, w[3][4 * i + 3], fmaf(z.z, w[3][4 * i + 2], fmaf(z.y, w[3][4 * i + 1], fmaf(z.x, w[3][4 * i], v.w))));
       }
     }
-    const float4 ps = bf16x4(__ldg(reinterpret_cast<const uint2*>(p.pos + static_cast<int64_t>(n) * p.d + c0)));
     *reinterpret_cast<float4*>(p.h + static_cast<int64_t>(r) * p.d + c0) =
         make_float4(v.x + ps.x, v.y + ps.y, v.z + ps.z, v.w + ps.w);
   }
@@ -652,8 +654,8 @@ __device__ __forceinline__ void gemv_store(const GemvParams& p, float* out, int 
   if (p.out_silu) p.out_silu[static_cast<int64_t>(r) * p.ldo + j] = silu_f(v);
 }
 
-// COLS columns per warp: 32 / RMAX with several rows; for one row 4, or 1 where the columns are
-// too few to fill the SMs otherwise (the conditioning MLP: 1152 columns).
+// COLS columns per warp: 32 / RMAX with several rows, 4 with one; 1 where the columns are too few
+// to fill the SMs otherwise (the conditioning MLP: 1152 columns, the head's modulation: 2304).
 template <int RMAX, int COLS>
 __global__ void __launch_bounds__(256) gemv_kernel(const GemvParams p) {
   extern __shared__ float xs[];  // [xrows][2 planes][K / 2]
@@ -741,7 +743,21 @@ __global__ void __launch_bounds__(256) gemv_kernel(const GemvParams p) {
     float acc[kCols * RMAX];
 #pragma unroll
     for (int i = 0; i < kCols * RMAX; ++i) acc[i] = sum_f32x2(acc2[i]);
-    if constexpr (kCols * RMAX == 32) {
+    if constexpr (kCols * RMAX == 8) {  // one column: lanes 4 i .. 4 i + 3 end with row i
+#pragma unroll
+      for (int o = 16; o >= 4; o >>= 1) {
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o / 4; ++i) {
+          const float send = upper ? acc[i] : acc[i + o / 4];
+          acc[i] = (upper ? acc[i + o / 4] : acc[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      float v = acc[0];
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      if ((lane & 3) == 0 && (lane >> 2) < p.rows) gemv_store(p, out, lane >> 2, j0, v);
+    } else if constexpr (kCols * RMAX == 32) {
       // lane l: column j0 + l / RMAX, row l % RMAX
       const float v = transpose_reduce32(acc, lane);
       const int c = lane / RMAX, r = lane % RMAX;
@@ -1149,8 +1165,8 @@ cudaError_t gemv_launch(const GemvParams& p, cudaStream_t s) {
       (p.n_seg > 0 && (p.out_silu || p.add_class || p.add_vec)) ||
       (p.ldx % 4) || (reinterpret_cast<uintptr_t>(p.x) & 15u))
     return cudaErrorInvalidValue;
+  const bool few = static_cast<int64_t>(p.N) * std::max(p.n_seg, 1) < 32ll * num_sms();
   if (xrows == 1) {
-    const bool few = static_cast<int64_t>(p.N) * std::max(p.n_seg, 1) < 64ll * num_sms();
     return few ? gemv_launch_r<1, 1>(p, smem, s) : gemv_launch_r<1, 4>(p, smem, s);
   }
   // many columns of a wide-enough weight to keep every SM streaming, and buffers that fit
@@ -1162,7 +1178,7 @@ cudaError_t gemv_launch(const GemvParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     return launch_k(gemv_stream_kernel, dim3(num_sms()), dim3(kStreamThreads), bytes, s, p, device_status_ptr());
   }
-  if (xrows <= 8) return gemv_launch_r<8, 4>(p, smem, s);
+  if (xrows <= 8) return few ? gemv_launch_r<8, 1>(p, smem, s) : gemv_launch_r<8, 4>(p, smem, s);
   return gemv_launch_r<16, 2>(p, smem, s);
 }
 

@@ -157,8 +157,15 @@ __device__ __forceinline__ void group_epilogue(const TcArgs& a, void* out, int r
         if (kOut % 32 != 0 && cc >= kOut) break;
         float x[16], y[16];
         src.load2(cc, kOut + cc, x, y);
+        if (e.act) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = e.act ? x[i] * gelu_erf_f(y[i]) : silu_f(x[i]) * y[i];
+          for (int i = 0; i < 16; ++i) x[i] *= gelu_erf_f(y[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) silu2(x[i], x[i + 1]);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) x[i] *= y[i];
+        }
         stage_put16_f16(stg, half, x);
       }
       stage_flush_f16(e, out, row0, a.M, min(a.N, n0 + kOut), n0 + c, stg);
@@ -174,9 +181,12 @@ __device__ __forceinline__ void group_epilogue(const TcArgs& a, void* out, int r
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         float* v = half ? y : x;
-        if (e.kind == SGD_EPI_GELU) {
+        if (e.kind == SGD_EPI_GELU && e.act) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = e.act ? gelu_erf_f(v[i]) : gelu_tanh_f(v[i]);
+          for (int i = 0; i < 16; ++i) v[i] = gelu_erf_f(v[i]);
+        } else if (e.kind == SGD_EPI_GELU) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) gelu_tanh2(v[i], v[i + 1]);
         }
         if (e.kind == SGD_EPI_F32)
           stage_put16_f32(stg, half, v);
