@@ -266,6 +266,32 @@ __device__ __forceinline__ uint32_t pack_f16x2_rn(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// The softmax of a query row in registers, where a thread's own instructions are the longest
+// part of the chain S -> P -> O: three-input maxima and paired multiplications and additions.
+template <int N>
+__device__ __forceinline__ float row_max(const uint32_t* r) {
+  float mx[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) mx[i] = fmaxf(__uint_as_float(r[i]), __uint_as_float(r[i + 8]));
+#pragma unroll
+  for (int c = 16; c < N; c += 16)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mx[i] = max3(mx[i], __uint_as_float(r[c + i]), __uint_as_float(r[c + 8 + i]));
+  return fmaxf(max3(mx[0], mx[1], mx[2]), max3(max3(mx[3], mx[4], mx[5]), mx[6], mx[7]));
+}
+
+// P = 2^(score * scale - m2) of 32 scores, packed in place as fp16 pairs (pair k into register k, its
+// scores already used), and their sums added to `sum` (four chains of pairs).
+__device__ __forceinline__ void exp_pack32(uint32_t* r, uint64_t scale2, uint64_t neg_m2, uint64_t* sum) {
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const uint64_t t = fma_f32x2(pack_f32x2(r[2 * k], r[2 * k + 1]), scale2, neg_m2);
+    const float p0 = ex2_approx(lo_f32x2(t)), p1 = ex2_approx(hi_f32x2(t));
+    sum[k & 3] = add_f32x2(sum[k & 3], pack_f32x2(p0, p1));
+    r[k] = pack_f16x2_rn(p0, p1);
+  }
+}
+
 struct AttnTcArgs {
   CUtensorMap tmap_q;
   CUtensorMap tmap_k;
@@ -538,8 +564,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
 // attn_pp_kernel: two query tiles per CTA, ping-pong between two softmax warpgroups.
 //
 // One CTA = 256 queries (tiles 0 and 1) of one (sample, head); K/V tiles of 128 keys, shared
-// by both query tiles, through a 2-stage TMA ring.  TMEM holds S_0, S_1 (128 fp32 columns
-// each) and O_0, O_1 (d_h columns each).  Warps 2-5 run the softmax of tile 0, warps 6-9 of
+// by both query tiles, through a 2-stage TMA ring in which K and V have their own barriers: the
+// K of tile j + 2 is fetched once S_1(j) has read K(j), not only after P V_1(j) (with one
+// barrier for both, S_0(j + 1) waited 600 to 800 of the 3300 clocks of a key tile for it at d_h
+// 128).  TMEM holds S_0, S_1 (128 fp32 columns each) and O_0, O_1 (d_h columns each).  Warps 2-5 run the softmax of tile 0, warps 6-9 of
 // tile 1: each reads its S from TMEM (a max pass, then an exp pass), writes P as fp16 pairs
 // over the first 64 columns of the same S, and the MMA warp computes O_t += P_t V from
 // Tensor Memory (A operand in TMEM), so P needs no shared memory.  The MMA warp issues, per
@@ -583,13 +611,16 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kBar);
   uint64_t* q_full = bars;
-  uint64_t* kv_full = bars + 1;
-  uint64_t* kv_empty = bars + 3;
+  uint64_t* k_full = bars + 1;
+  uint64_t* k_empty = bars + 3;
   uint64_t* s_full = bars + 5;   // per query tile
-  uint64_t* p_full = bars + 7;   // per query tile, 4 warps arrive
+  uint64_t* p_lo = bars + 7;     // per query tile, 4 warps arrive: P of the first 64 keys
   uint64_t* o_done = bars + 9;   // per query tile
   uint64_t* drain = bars + 11;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+  uint64_t* p_hi = bars + 12;    // ... and of the other 64
+  uint64_t* v_full = bars + 14;
+  uint64_t* v_empty = bars + 16;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -603,10 +634,13 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&kv_full[i], 1);
-      mbar_init(&kv_empty[i], 1);
+      mbar_init(&k_full[i], 1);
+      mbar_init(&k_empty[i], 1);
+      mbar_init(&v_full[i], 1);
+      mbar_init(&v_empty[i], 1);
       mbar_init(&s_full[i], 1);
-      mbar_init(&p_full[i], 4);
+      mbar_init(&p_lo[i], 4);
+      mbar_init(&p_hi[i], 4);
       mbar_init(&o_done[i], 1);
     }
     mbar_init(drain, 1);
@@ -628,7 +662,8 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
 
   if (warp == 0) {
     const bool lead = elect_one();
-    const uint32_t sm0 = smem_u32(sm), kv_full0 = smem_u32(kv_full), kv_empty0 = smem_u32(kv_empty);
+    const uint32_t sm0 = smem_u32(sm), k_full0 = smem_u32(k_full), k_empty0 = smem_u32(k_empty);
+    const uint32_t v_full0 = smem_u32(v_full), v_empty0 = smem_u32(v_empty);
     const int col0 = h * a.head_stride;
     // one 128-row operand tile: its 64-column atoms, then (d_h 72) its 16-column atom
     auto load_tile = [&](uint32_t dst, const CUtensorMap* m64, const CUtensorMap* m16, uint32_t bar, int row) {
@@ -644,18 +679,27 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
     int j = 0;
     for (; j < nt; ++j) {
       const int s = j & 1;
-      if (!mbar_wait_warp(kv_empty0 + 8 * s, ((j >> 1) & 1) ^ 1u, abort_flag, a.status, 21)) break;
+      const uint32_t ph = ((j >> 1) & 1) ^ 1u, st = sm0 + L::kKV + s * L::kStage;
+      const int row = b * a.n_kv + j * kTcBK;
+      if (!mbar_wait_warp(k_empty0 + 8 * s, ph, abort_flag, a.status, 21)) break;
       if (lead) {
-        const uint32_t st = sm0 + L::kKV + s * L::kStage, bar = kv_full0 + 8 * s;
-        mbar_arrive_expect_tx_at(bar, 2 * L::kTile);
-        const int row = b * a.n_kv + j * kTcBK;
-        load_tile(st, &a.tmap_k, &a.tmap_k16, bar, row);
-        load_tile(st + L::kTile, &a.tmap_v, &a.tmap_v16, bar, row);
+        mbar_arrive_expect_tx_at(k_full0 + 8 * s, L::kTile);
+        load_tile(st, &a.tmap_k, &a.tmap_k16, k_full0 + 8 * s, row);
+      }
+      if (!mbar_wait_warp(v_empty0 + 8 * s, ph, abort_flag, a.status, 20)) break;
+      if (lead) {
+        mbar_arrive_expect_tx_at(v_full0 + 8 * s, L::kTile);
+        load_tile(st + L::kTile, &a.tmap_v, &a.tmap_v16, v_full0 + 8 * s, row);
       }
     }
     if (lead && *abort_flag) {
       mbar_drain(q_full, 0);
-      for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) mbar_drain(&kv_full[i & 1], (i >> 1) & 1);
+      // (a K tile whose V tile was not asked for any more is the j-th)
+      for (int i = (j > 2 ? j - 2 : 0); i < j; ++i) {
+        mbar_drain(&k_full[i & 1], (i >> 1) & 1);
+        mbar_drain(&v_full[i & 1], (i >> 1) & 1);
+      }
+      if (j < nt) mbar_drain(&k_full[j & 1], (j >> 1) & 1);
     }
   } else if (warp == 1) {
     // The whole warp runs the loop, one elected lane issues, and every operand of an MMA is a
@@ -665,8 +709,9 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
     constexpr uint32_t idesc_qk = umma_idesc_f16(kTcBQ, kTcBK);
     constexpr uint32_t idesc_pv = umma_idesc_f16_bmn(kTcBQ, 64 * L::kA64);
     constexpr uint32_t idesc_pv16 = umma_idesc_f16_bmn(kTcBQ, 16);
-    const uint32_t sm0 = smem_u32(sm), kv_full0 = smem_u32(kv_full), kv_empty0 = smem_u32(kv_empty);
-    const uint32_t s_full0 = smem_u32(s_full), p_full0 = smem_u32(p_full), o_done0 = smem_u32(o_done);
+    const uint32_t sm0 = smem_u32(sm), k_full0 = smem_u32(k_full), k_empty0 = smem_u32(k_empty);
+    const uint32_t v_full0 = smem_u32(v_full), v_empty0 = smem_u32(v_empty);
+    const uint32_t s_full0 = smem_u32(s_full), p_lo0 = smem_u32(p_lo), p_hi0 = smem_u32(p_hi), o_done0 = smem_u32(o_done);
     const uint64_t dq = smem_desc_sw128(sm0 + L::kQ), dk = smem_desc_sw128(sm0 + L::kKV);
     const uint64_t dv = smem_desc_sw128_mn(sm0 + L::kKV + L::kTile, kAtom, 1024);
     const uint64_t dq16 = smem_desc_sw32(sm0 + L::kQ + L::kA64 * kAtom);
@@ -687,41 +732,51 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
         umma_f16(d, dq16 + t * kTileU, dk16 + s * kStageU, idesc_qk, 1u);
       umma_commit_at(s_full0 + 8 * t);
     };
-    auto issue_pv = [&](int t, int s, uint32_t accumulate) {
+    // O_t (+)= P_t V over the 64 keys of one half, as soon as their P is there
+    auto pv_half = [&](int t, int s, int half, uint32_t accumulate) {
       if (!lead) return;
       const uint32_t pa = tmem + L::kTmemS + t * kTcBK, d = tmem + L::kTmemO + t * L::kDP;
       const uint64_t va = dv + s * kStageU, va16 = dv16 + s * kStageU;
 #pragma unroll
-      for (int ks = 0; ks < kTcBK / 16; ++ks) {
-        umma_f16_ts(d, pa + 8 * ks, va + ks * (2048 >> 4), idesc_pv, ks > 0 ? 1u : accumulate);
+      for (int i = 0; i < kTcBK / 32; ++i) {
+        const int ks = half * (kTcBK / 32) + i;
+        umma_f16_ts(d, pa + 8 * ks, va + ks * (2048 >> 4), idesc_pv, i > 0 ? 1u : accumulate);
         if (L::kPad)  // O columns 64..79 from the 16-column V atom (8-key-row groups 256 B apart)
-          umma_f16_ts(d + 64 * L::kA64, pa + 8 * ks, va16 + ks * (512 >> 4), idesc_pv16, ks > 0 ? 1u : accumulate);
+          umma_f16_ts(d + 64 * L::kA64, pa + 8 * ks, va16 + ks * (512 >> 4), idesc_pv16, i > 0 ? 1u : accumulate);
       }
-      umma_commit_at(o_done0 + 8 * t);
+      if (half) umma_commit_at(o_done0 + 8 * t);
     };
-    if (ok && (ok = mbar_wait_warp(kv_full0, 0, abort_flag, a.status, 23))) {
+    auto issue_pv = [&](int t, int s, uint32_t ph, uint32_t accumulate) -> bool {
+      if (!mbar_wait_warp(p_lo0 + 8 * t, ph, abort_flag, a.status, 24 + 2 * t)) return false;
+      tc_fence_after();
+      pv_half(t, s, 0, accumulate);
+      if (!mbar_wait_warp(p_hi0 + 8 * t, ph, abort_flag, a.status, 24 + 2 * t)) return false;
+      tc_fence_after();
+      pv_half(t, s, 1, 1u);
+      return true;
+    };
+    if (ok && (ok = mbar_wait_warp(k_full0, 0, abort_flag, a.status, 23))) {
       tc_fence_after();
       issue_qk(0, 0);
       if (two) issue_qk(1, 0);
+      if (lead) umma_commit_at(k_empty0);
     }
     for (int j = 0; j < nt && ok; ++j) {
       const int s = j & 1;
       const uint32_t ph = j & 1, acc = j > 0 ? 1u : 0u;
-      if (!(ok = mbar_wait_warp(p_full0, ph, abort_flag, a.status, 24))) break;
-      tc_fence_after();
-      issue_pv(0, s, acc);
+      if (!(ok = mbar_wait_warp(v_full0 + 8 * s, (j >> 1) & 1, abort_flag, a.status, 30))) break;
+      if (!(ok = issue_pv(0, s, ph, acc))) break;
       if (j + 1 < nt) {
-        if (!(ok = mbar_wait_warp(kv_full0 + 8 * (s ^ 1), ((j + 1) >> 1) & 1, abort_flag, a.status, 25))) break;
+        if (!(ok = mbar_wait_warp(k_full0 + 8 * (s ^ 1), ((j + 1) >> 1) & 1, abort_flag, a.status, 25))) break;
         tc_fence_after();
         issue_qk(0, s ^ 1);
       }
-      if (two) {
-        if (!(ok = mbar_wait_warp(p_full0 + 8, ph, abort_flag, a.status, 26))) break;
-        tc_fence_after();
-        issue_pv(1, s, acc);
+      if (two && !(ok = issue_pv(1, s, ph, acc))) break;
+      if (lead) umma_commit_at(v_empty0 + 8 * s);
+      if (j + 1 < nt) {
+        if (two) issue_qk(1, s ^ 1);
+        if (lead) umma_commit_at(k_empty0 + 8 * (s ^ 1));
       }
-      if (lead) umma_commit_at(kv_empty0 + 8 * s);
-      if (two && j + 1 < nt) issue_qk(1, s ^ 1);
     }
     if (lead) {
       umma_commit(drain);
@@ -753,13 +808,7 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
           if (c >= nvalid) r[c] = __float_as_uint(-INFINITY);
       }
       // the row maximum of the raw scores (scale > 0 commutes with max), then log2 units
-      float mx[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) mx[i] = __uint_as_float(r[i]);
-#pragma unroll
-      for (int c = 8; c < kTcBK; ++c) mx[c & 7] = fmaxf(mx[c & 7], __uint_as_float(r[c]));
-      const float mt = a.scale_log2 * fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
-                                            fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
+      const float mt = a.scale_log2 * row_max<kTcBK>(r);
       if (j == 0) {
         m2 = mt;
       } else if (__any_sync(0xffffffffu, mt > m2 + kRescaleLog2)) {
@@ -781,29 +830,23 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
         l *= corr;
         m2 = mnew;
       }
-      // P = 2^(score * scale - m2) packed as fp16 pairs in place (pair k of a 32-score chunk
-      // into register k of the chunk, already consumed) and stored over columns [0, 64) of
-      // this S: chunk c's 16 packed columns land on scores already read
-      const float neg_m2 = -m2;
-      float ls[8];
+      // P as fp16 pairs, stored over columns [0, 64) of this S (chunk c's 16 packed columns land on
+      // scores already read); the MMA warp starts on the first 64 keys while the others follow
+      const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2), neg_m2 = pack_f32x2(-m2, -m2);
+      uint64_t sum[4] = {0, 0, 0, 0};
 #pragma unroll
-      for (int i = 0; i < 8; ++i) ls[i] = 0.f;
+      for (int half = 0; half < 2; ++half) {
 #pragma unroll
-      for (int c = 0; c < kTcBK; c += 32) {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          const float p0 = ex2_approx(fmaf(__uint_as_float(r[c + 2 * k]), a.scale_log2, neg_m2));
-          const float p1 = ex2_approx(fmaf(__uint_as_float(r[c + 2 * k + 1]), a.scale_log2, neg_m2));
-          ls[k & 7] += p0 + p1;
-          r[c + k] = pack_f16x2_rn(p0, p1);
+        for (int c = 64 * half; c < 64 * half + 64; c += 32) {
+          exp_pack32(r + c, scale2, neg_m2, sum);
+          tmem_st16(s_col + c / 2, r + c);
         }
-        tmem_st16(s_col + c / 2, r + c);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(half ? &p_hi[t] : &p_lo[t]);
       }
-      l += ((ls[0] + ls[1]) + (ls[2] + ls[3])) + ((ls[4] + ls[5]) + (ls[6] + ls[7]));
-      tmem_st_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_full[t]);
+      l += sum_f32x2(add_f32x2(add_f32x2(sum[0], sum[1]), add_f32x2(sum[2], sum[3])));
     }
     if (ok && mbar_wait_warp(smem_u32(&o_done[t]), (nt - 1) & 1, abort_flag, a.status, 29)) {
       tc_fence_after();
@@ -1020,12 +1063,7 @@ __global__ void __launch_bounds__(kSmThreads, SmLayout<DH>::kBlocks) attn_sm_ker
           for (int c = 0; c < kSmBK; ++c)
             if (c >= nvalid) r[c] = __float_as_uint(-INFINITY);
         }
-        float mx[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) mx[i] = __uint_as_float(r[i]);
-#pragma unroll
-        for (int c = 4; c < kSmBK; ++c) mx[c & 3] = fmaxf(mx[c & 3], __uint_as_float(r[c]));
-        const float mt = a.scale_log2 * fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        const float mt = a.scale_log2 * row_max<kSmBK>(r);
         if (j == 0) {
           m2 = mt;
         } else if (__any_sync(0xffffffffu, mt > m2 + kRescaleLog2)) {
@@ -1047,22 +1085,14 @@ __global__ void __launch_bounds__(kSmThreads, SmLayout<DH>::kBlocks) attn_sm_ker
           l *= corr;
           m2 = mnew;
         }
-        const float neg_m2 = -m2;
-        float ls[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) ls[i] = 0.f;
+        const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2), neg_m2 = pack_f32x2(-m2, -m2);
+        uint64_t sum[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int c = 0; c < kSmBK; c += 32) {
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const float p0 = ex2_approx(fmaf(__uint_as_float(r[c + 2 * k]), a.scale_log2, neg_m2));
-            const float p1 = ex2_approx(fmaf(__uint_as_float(r[c + 2 * k + 1]), a.scale_log2, neg_m2));
-            ls[k & 3] += p0 + p1;
-            r[c + k] = pack_f16x2_rn(p0, p1);
-          }
+          exp_pack32(r + c, scale2, neg_m2, sum);
           tmem_st16(s_col + c / 2, r + c);
         }
-        l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        l += sum_f32x2(add_f32x2(add_f32x2(sum[0], sum[1]), add_f32x2(sum[2], sum[3])));
         tmem_st_wait();
       }
       tc_fence_before();

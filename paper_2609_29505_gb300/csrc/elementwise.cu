@@ -617,18 +617,6 @@ __global__ void stem_patch_any_kernel(const StemParams p) {
 // The products are formed as pairs of even and odd k (fma.rn.f32x2, two fp32 fmas per
 // instruction, both halves added at the end): with one fma per instruction and 8 rows the fma
 // pipe came close to the weight stream's time.
-__device__ __forceinline__ uint64_t pack_f32x2(uint32_t lo, uint32_t hi) {
-  uint64_t d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
-  return d;
-}
-__device__ __forceinline__ void fma_f32x2(uint64_t& d, uint64_t a, uint64_t b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ float sum_f32x2(uint64_t a) {
-  return __uint_as_float(static_cast<uint32_t>(a)) + __uint_as_float(static_cast<uint32_t>(a >> 32));
-}
-
 // v[0..31] of every lane -> lane l returns the warp's sum of value l
 __device__ __forceinline__ float transpose_reduce32(float* v, int lane) {
 #pragma unroll
@@ -736,7 +724,7 @@ __global__ void __launch_bounds__(256) gemv_kernel(const GemvParams p) {
 #pragma unroll
           for (int c = 0; c < kCols; ++c)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) fma_f32x2(acc2[c * RMAX + r], wf[c][q], xv[q]);
+            for (int q = 0; q < 4; ++q) acc2[c * RMAX + r] = fma_f32x2(wf[c][q], xv[q], acc2[c * RMAX + r]);
         }
       }
     }
@@ -860,7 +848,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) gemv_stream_kernel(const Ge
 #pragma unroll
         for (int c = 0; c < 4; ++c)
 #pragma unroll
-          for (int q = 0; q < 4; ++q) fma_f32x2(acc2[c * 8 + r], wf[c][q], xv[q]);
+          for (int q = 0; q < 4; ++q) acc2[c * 8 + r] = fma_f32x2(wf[c][q], xv[q], acc2[c * 8 + r]);
       }
     }
     __syncwarp();
