@@ -256,19 +256,28 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// A wait looks at the abort flag and at %globaltimer (whose read stalls the reading thread for
+// hundreds of clocks) once in kPollsPerTimer polls, so that a wait of the usual length only polls.
+constexpr uint32_t kPollsPerTimer = 256;
+
+__device__ __forceinline__ bool wait_expired(uint64_t& t0) {
+  const uint64_t now = global_timer_ns();
+  if (t0 == 0) t0 = now;
+  return now - t0 > kWaitTimeoutNs;
+}
+
 // Wait for the phase with parity `parity` of `bar` to complete.  Returns false (and
 // leaves the barrier alone) if the CTA-wide abort flag is raised or the wait exceeds
 // kWaitTimeoutNs; in the latter case it raises the flag and records `code` in
 // *status.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           int* status, int code) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_timer_ns();
+  uint64_t t0 = 0;
   for (uint32_t i = 1;; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 31u) == 0u) {
+    if (i % kPollsPerTimer == 0) {
       if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > kWaitTimeoutNs) {
+      if (wait_expired(t0)) {
         *abort_flag = 1;
         if (status) atomicCAS(status, 0, code);
         return false;
@@ -293,13 +302,12 @@ __device__ __forceinline__ bool mbar_try_wait_at(uint32_t bar, uint32_t parity) 
 
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                                int* status, int code) {
-  if (__all_sync(0xffffffffu, mbar_try_wait_at(bar, parity))) return true;
-  const uint64_t t0 = global_timer_ns();
+  uint64_t t0 = 0;
   for (uint32_t i = 1;; ++i) {
     if (__all_sync(0xffffffffu, mbar_try_wait_at(bar, parity))) return true;
-    if ((i & 31u) == 0u) {
+    if (i % kPollsPerTimer == 0) {
       int stop = *abort_flag;
-      if (!stop && global_timer_ns() - t0 > kWaitTimeoutNs) {
+      if (!stop && wait_expired(t0)) {
         *abort_flag = stop = 1;
         if (status) atomicCAS(status, 0, code);
       }
