@@ -3,6 +3,7 @@
 // word and the fixed scratch of the allocation-free entry.  The kernel itself is in
 // gemm_kernel.cuh.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -181,10 +182,14 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 }  // namespace
 
 int num_sms() {
+  static std::atomic<int> sms[64];  // per device, 0 until asked for
   int dev = 0, n = 0;
-  cudaGetDevice(&dev);
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+  if ((n = sms[dev].load(std::memory_order_relaxed)) > 0) return n;
   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-  return n > 0 ? n : 1;
+  n = n > 0 ? n : 1;
+  sms[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // ----------------------------------------------------------------------------
