@@ -285,7 +285,9 @@ SkSplit sk_split(int num_tiles, int num_k, int sms, bool force = false) {
 // Tile of the CTA-group kernel (sets p.group, p.bn).  In SM clocks, a launch takes about
 //   waves x (K-blocks x time of a K-block + kWave) + the last tile's epilogue (+ kPair),
 // a K-block a little over 2 BN on the tensor cores, or the issue loop's 324, unless its operand
-// bytes take longer to reach the SM (kRate per clock with all SMs loading).  The constants are
+// bytes take longer through shared memory, which TMA writes once and the MMAs read once (kRate
+// operand bytes per clock; write and read together are 124 to 150 in every tile measured, and
+// sharing A between two CTAs by TMA multicast changed nothing).  The constants are
 // fitted to graph-replayed launches of 46 shapes, of which the chosen tile is within 5% of the best
 // (us; a CTA's 128 x 64, 128, 256 / a pair's 256 x 128, 160, 192, 224, 256):
 //   64 x 256 x 256 residual       4.7   5.8   9.1 /

@@ -4,9 +4,9 @@
 // CG = 2: a cluster of two CTAs computes one 256 x BN output tile (tcgen05 cta_group::2).  Each CTA
 // loads its own 128 rows of A and half of B's BN rows per 64-wide K-block (16 KB + BN * 64 bytes),
 // and the leader's tcgen05.mma (M = 256) reads both CTAs' shared memory and accumulates 128 rows
-// in each CTA's TMEM.  A 1-CTA tile of 128 x 256 needs 48 KB per K-block for 512 tensor-core
-// clocks, above the ~70 bytes per clock that reach an SM from L2 when all of them load; the pair
-// needs 32 KB.  CG = 1: a CTA computes a 128 x BN tile by itself, for problems of few rows.
+// in each CTA's TMEM.  A 1-CTA tile of 128 x 256 puts 48 KB per K-block into shared memory and
+// reads them back in 512 tensor-core clocks, more than shared memory moves (it takes 692); the
+// pair puts 32 KB there (528).  CG = 1: a CTA computes a 128 x BN tile by itself, for problems of few rows.
 // One epilogue per instantiation keeps every value of it in registers (the kernel that holds
 // all of them in one body spills) and the code that a short launch has to fetch small.
 //
