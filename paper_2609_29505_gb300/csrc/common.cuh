@@ -215,7 +215,8 @@ __device__ __forceinline__ uint32_t lane_id() {
 // (returns at once for a grid launched without programmatic serialization), then let the
 // next grid in the stream begin launching (its CTAs run their own prologue and wait here in
 // turn).  Every kernel of a step program calls this after its shared-memory / TMEM-only
-// prologue and before its first global-memory access.
+// prologue and before its first global-memory access (but for the group GEMM's first loads of
+// its weight, which no kernel of a step program writes).
 __device__ __forceinline__ void pdl_wait_and_trigger() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
