@@ -48,36 +48,70 @@ struct GroupCfg {
   static_assert((2 * kStages + 5) * 8 + 4 * 4 <= 512, "barrier block");
 };
 
+// cos and sin of 4 pairs of each of a lane's 4 rows, and where the rows' tables start (-1: no row).
+struct RopeTab {
+  int64_t at[4];
+  float4 cs[4], sn[4];
+};
+__device__ __forceinline__ void rope_load(const EpiParams& e, bool rot, int j, RopeTab& t) {
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    if (rot && t.at[it] >= 0) {
+      t.cs[it] = *reinterpret_cast<const float4*>(e.rope_cos + t.at[it] + j);
+      t.sn[it] = *reinterpret_cast<const float4*>(e.rope_sin + t.at[it] + j);
+    }
+  }
+}
+
+// Column range cb .. ce and pairs j0 .. j1 of every head that a warp's half of a tile covers: whole
+// heads, or half of the pairs of the tile's one head.
+template <int BN>
+struct RopeRange {
+  int cb, ce, j0, j1;
+  __device__ __forceinline__ RopeRange(int hd, int part) {
+    const bool heads = 2 * hd <= BN / 2;
+    cb = heads && part ? BN / 2 : 0;
+    ce = heads && !part ? BN / 2 : BN;
+    j0 = !heads && part ? hd / 2 : 0;
+    j1 = !heads && !part ? hd / 2 : hd;
+  }
+};
+
+// The tables of the first chunk, which the accumulator is not needed for.
+template <int BN>
+__device__ __forceinline__ void rope_begin(const TcArgs& a, int row0, int n0, int part, RopeTab& t) {
+  const int lane = threadIdx.x & 31, hd = a.epi.d_head >> 1;
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const int r = row0 + it * 8 + (lane >> 2);
+    t.at[it] = r < a.M ? static_cast<int64_t>(r % a.epi.rope_tokens) * hd + 4 * (lane & 3) : -1;
+  }
+  const RopeRange<BN> g(hd, part);
+  rope_load(a.epi, n0 + g.cb < a.epi.rope_cols, g.j0, t);
+}
+
 // RoPE through the staging buffer: 16 columns of a head's first half and the 16 they rotate
 // with go through shared memory together, and each lane rotates 4 pairs of a row, with cos and
-// sin read 64 bytes per row.
-template <class Src>
-__device__ __forceinline__ void rope_staged(const TcArgs& a, void* out, int row, int n0, const Src& src, int cb,
-                                            int ce, int j0, int j1, float4* stg) {
+// sin read 64 bytes per row.  The first chunk's tables are fetched before the accumulator is there
+// and the next chunk's while one is rotated (read when a chunk needed them, each of a warp's 4
+// chunks waited for L2: 64 x 768 x 256 6.65 -> 5.80 us, 333 x 12288 x 256 10.8 -> 9.9,
+// 333 x 12288 x 4096 34.1 -> 32.9).
+template <int BN, class Src>
+__device__ __forceinline__ void rope_staged(const TcArgs& a, void* out, int row, int n0, const Src& src, int part,
+                                            float4* stg, RopeTab& t) {
   const EpiParams& e = a.epi;
   const int lane = threadIdx.x & 31;
   const int row0 = row - lane;
   const int lr = lane >> 2, lc = lane & 3;
-  const int dh = e.d_head, hd = dh >> 1;  // pairs j0 .. j1 - 1 of the heads at columns cb .. ce - 1
+  const int dh = e.d_head, hd = dh >> 1;
+  const RopeRange<BN> g(hd, part);
   f16* o = reinterpret_cast<f16*>(out);
 #pragma unroll 1
-  for (int hb = cb; hb < ce; hb += dh) {
+  for (int hb = g.cb; hb < g.ce; hb += dh) {
     if (n0 + hb >= a.N) break;  // N is a multiple of d_head or the head's columns are checked below
     const bool rot = n0 + hb < e.rope_cols;
 #pragma unroll 1
-    for (int j = j0; j < j1; j += 16) {
-      float4 cs[4], sn[4];
-#pragma unroll
-      for (int it = 0; it < 4; ++it) {
-        cs[it] = make_float4(1.f, 1.f, 1.f, 1.f);
-        sn[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int r = row0 + it * 8 + lr;
-        if (rot && r < a.M) {
-          const int64_t at = static_cast<int64_t>(r % e.rope_tokens) * hd + j + 4 * lc;
-          cs[it] = *reinterpret_cast<const float4*>(e.rope_cos + at);
-          sn[it] = *reinterpret_cast<const float4*>(e.rope_sin + at);
-        }
-      }
+    for (int j = g.j0; j < g.j1; j += 16) {
       {
         float x[16], y[16];
         src.load2(hb + j, hb + hd + j, x, y);
@@ -85,6 +119,11 @@ __device__ __forceinline__ void rope_staged(const TcArgs& a, void* out, int row,
         stage_put16_f32(stg, 1, y);
       }
       __syncwarp();
+      const RopeTab c = t;
+      if (j + 16 < g.j1)
+        rope_load(e, rot, j + 16, t);
+      else if (hb + dh < g.ce)
+        rope_load(e, n0 + hb + dh < e.rope_cols, g.j0, t);
       const int c1 = n0 + hb + j + 4 * lc, c2 = c1 + hd;
 #pragma unroll
       for (int it = 0; it < 4; ++it) {
@@ -92,9 +131,9 @@ __device__ __forceinline__ void rope_staged(const TcArgs& a, void* out, int row,
         const float4 p = stg[r * 8 + (lc ^ (r & 7))], q = stg[r * 8 + ((lc + 4) ^ (r & 7))];
         float4 u = p, v = q;
         if (rot) {
-          const float4 c = cs[it], s = sn[it];
-          u = make_float4(p.x * c.x - q.x * s.x, p.y * c.y - q.y * s.y, p.z * c.z - q.z * s.z, p.w * c.w - q.w * s.w);
-          v = make_float4(q.x * c.x + p.x * s.x, q.y * c.y + p.y * s.y, q.z * c.z + p.z * s.z, q.w * c.w + p.w * s.w);
+          const float4 cs = c.cs[it], s = c.sn[it];
+          u = make_float4(p.x * cs.x - q.x * s.x, p.y * cs.y - q.y * s.y, p.z * cs.z - q.z * s.z, p.w * cs.w - q.w * s.w);
+          v = make_float4(q.x * cs.x + p.x * s.x, q.y * cs.y + p.y * s.y, q.z * cs.z + p.z * s.z, q.w * cs.w + p.w * s.w);
         }
         if (row0 + r < a.M) {
           f16* orow = o + static_cast<int64_t>(row0 + r) * e.ldo;
@@ -131,7 +170,7 @@ __device__ __forceinline__ void arrive_leader(uint32_t bar) {
 
 template <int BN, int EP, class Src>
 __device__ __forceinline__ void group_epilogue(const TcArgs& a, void* out, int row, int n_blk, const Src& src,
-                                              int part, float4* stg, float4* hv) {
+                                              int part, float4* stg, float4* hv, RopeTab& rt) {
   const EpiParams& e = a.epi;
   const int row0 = row - (threadIdx.x & 31);
   if constexpr (EP == kEpDelta) {
@@ -139,12 +178,7 @@ __device__ __forceinline__ void group_epilogue(const TcArgs& a, void* out, int r
     delta_staged<true>(a, row, n_blk * BN, src, part ? kSplit : 0, part ? BN : kSplit,
                                                     stg, hv);
   } else if constexpr (EP == kEpRope) {
-    // the two column halves are whole heads, or halves of the tile's one head's pairs
-    const int hd = a.epi.d_head >> 1;
-    if (2 * hd <= BN / 2)
-      rope_staged(a, out, row, n_blk * BN, src, part ? BN / 2 : 0, part ? BN : BN / 2, 0, hd, stg);
-    else
-      rope_staged(a, out, row, n_blk * BN, src, 0, BN, part ? hd / 2 : 0, part ? hd : hd / 2, stg);
+    rope_staged<BN>(a, out, row, n_blk * BN, src, part, stg, rt);
   } else if constexpr (EP == kEpGated) {
     constexpr int kOut = BN / 2, kSplit = ((kOut / 32 + 1) / 2) * 32;
     const int n0 = n_blk * kOut, ce = part ? kOut : kSplit;
@@ -386,6 +420,7 @@ __device__ __forceinline__ void gemm_group_body(const TcArgs& a) {
     const uint32_t tempty0 = CG == 2 ? map_to_rank(smem_u32(tempty), 0) : smem_u32(tempty);
     void* out = a.epi.out_slot ? *a.epi.out_slot : a.epi.out;
     float4 hv[8];  // first 32-column chunk of h (delta_staged)
+    RopeTab rt;    // first chunk's tables (rope_staged)
     for (int tile = group, u = 0; tile < num_tiles; tile += num_groups, ++u) {
       int m_blk, n_blk;
       tile_coords(a, tile, m_blk, n_blk);
@@ -397,9 +432,10 @@ __device__ __forceinline__ void gemm_group_body(const TcArgs& a) {
         prefetch_h_row(a.epi, row, a.M, a.N, n_blk * BN, part ? kSplit : 0, part ? BN : kSplit);
         load_h_chunk(a, row - lane, n_blk * BN + (part ? kSplit : 0), hv);
       }
+      if (EP == kEpRope) rope_begin<BN>(a, row - lane, n_blk * BN, part, rt);
       if (!mbar_wait_warp(smem_u32(&tfull[acc]), aph, abort_flag, a.status, 34)) break;
       tc_fence_after();
-      group_epilogue<BN, EP>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, part, stg, hv);
+      group_epilogue<BN, EP>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, part, stg, hv, rt);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) arrive_leader<CG>(tempty0 + 8 * acc);
