@@ -582,7 +582,7 @@ def run_policies(binding, model, cfg, T, xs, out, cls, ctx, stream):
     return rows
 
 
-GEMM_SOURCES = ("gemm_kernel.cuh", "gemm.cu", "common.cuh")
+GEMM_SOURCES = ("gemm_group_kernel.cuh", "gemm_kernel.cuh", "gemm.cu", "common.cuh")
 
 
 def gemm_source_hash():
