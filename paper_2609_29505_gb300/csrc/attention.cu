@@ -885,6 +885,11 @@ __global__ void __launch_bounds__(kPpThreads, 1) attn_pp_kernel(const __grid_con
 // 64) or 256 columns of TMEM and 50 to 100 KB of shared memory: 3 (d_h 64) or 2 CTAs share an SM
 // and cover each other's latencies, ragged key counts waste at most 63 keys, and a warp whose 32
 // queries do not exist skips its softmax.  P overwrites S as in attn_pp_kernel.
+//
+// The first reference of a row is its maximum over 128 keys, as in attn_pp_kernel: with that of
+// 64 keys the largest probability of up to 128 keys was often not 1 but a rounded value above it
+// (77 keys: 2.40e-4 from float64 instead of 2.29e-4).  The scores of the second tile are formed
+// once more ahead of the loop, into O's columns, for their maxima alone.
 // ----------------------------------------------------------------------------
 constexpr int kSmThreads = 192;
 constexpr int kSmBK = 64;
@@ -998,21 +1003,23 @@ __global__ void __launch_bounds__(kSmThreads, SmLayout<DH>::kBlocks) attn_sm_ker
     const uint64_t dk16 = smem_desc_sw32(sm0 + L::kKV + L::kA64 * L::kAtomKV);
     const uint64_t dv16 = smem_desc_sw32_mn(sm0 + L::kKV + L::kTile + L::kA64 * L::kAtomKV, L::kAtomKV32, 256);
     constexpr uint64_t kStageU = L::kStage >> 4;
-    auto issue_qk = [&](int s) {
+    auto issue_qk = [&](uint32_t d, int s) {
       if (!lead) return;
       const uint64_t ka = dk + s * kStageU;
 #pragma unroll
       for (int ks = 0; ks < 4 * L::kA64; ++ks)
-        umma_f16(tmem, dq + (((ks >> 2) * kAtom + (ks & 3) * 32) >> 4),
+        umma_f16(d, dq + (((ks >> 2) * kAtom + (ks & 3) * 32) >> 4),
                  ka + (((ks >> 2) * L::kAtomKV + (ks & 3) * 32) >> 4), idesc_qk, ks > 0 ? 1u : 0u);
-      if (L::kPad) umma_f16(tmem, dq16, dk16 + s * kStageU, idesc_qk, 1u);  // head columns 64..79
-      umma_commit_at(smem_u32(s_full));
+      if (L::kPad) umma_f16(d, dq16, dk16 + s * kStageU, idesc_qk, 1u);  // head columns 64..79
     };
     bool ok = mbar_wait_warp(smem_u32(q_full), 0, abort_flag, a.status, 52) &&
               mbar_wait_warp(kv_full0, 0, abort_flag, a.status, 53);
+    if (ok && nt > 1) ok = mbar_wait_warp(kv_full0 + 8, 0, abort_flag, a.status, 53);
     if (ok) {
       tc_fence_after();
-      issue_qk(0);
+      issue_qk(tmem, 0);
+      if (nt > 1) issue_qk(tmem + L::kTmemO, 1);  // for its row maxima; PV(0) overwrites it
+      if (lead) umma_commit_at(smem_u32(s_full));
     }
     for (int j = 0; j < nt && ok; ++j) {
       const int s = j & 1;
@@ -1034,7 +1041,8 @@ __global__ void __launch_bounds__(kSmThreads, SmLayout<DH>::kBlocks) attn_sm_ker
       if (j + 1 < nt) {
         if (!(ok = mbar_wait_warp(kv_full0 + 8 * (s ^ 1), ((j + 1) >> 1) & 1, abort_flag, a.status, 55))) break;
         tc_fence_after();
-        issue_qk(s ^ 1);  // after PV(j) in issue order, which reads P where S goes
+        issue_qk(tmem, s ^ 1);  // after PV(j) in issue order, which reads P where S goes
+        if (lead) umma_commit_at(smem_u32(s_full));
       }
     }
     if (lead) {
@@ -1049,23 +1057,28 @@ __global__ void __launch_bounds__(kSmThreads, SmLayout<DH>::kBlocks) attn_sm_ker
     float m2 = -INFINITY, l = 0.f;
     bool ok = true;
     uint32_t r[kSmBK];
+    // the scores of key tile j from TMEM column `col` into r, and their maximum in log2 units
+    auto load_scores = [&](uint32_t col, int j) {
+      const int nvalid = min(a.n_kv - j * kSmBK, kSmBK);  // keys of this tile (the rest are masked)
+#pragma unroll
+      for (int c = 0; c < kSmBK; c += 16) tmem_ld16(col + c, r + c);
+#pragma unroll
+      for (int c = 0; c < kSmBK; c += 16) tmem_ld_wait16(r + c);
+      if (nvalid < kSmBK) {
+#pragma unroll
+        for (int c = 0; c < kSmBK; ++c)
+          if (c >= nvalid) r[c] = __float_as_uint(-INFINITY);
+      }
+      return a.scale_log2 * row_max<kSmBK>(r);
+    };
     for (int j = 0; j < nt && ok; ++j) {
       if (!(ok = mbar_wait_warp(smem_u32(s_full), j & 1, abort_flag, a.status, 56))) break;
       tc_fence_after();
       if (any) {
-        const int nvalid = min(a.n_kv - j * kSmBK, kSmBK);  // keys of this tile (the rest are masked)
-#pragma unroll
-        for (int c = 0; c < kSmBK; c += 16) tmem_ld16(s_col + c, r + c);
-#pragma unroll
-        for (int c = 0; c < kSmBK; c += 16) tmem_ld_wait16(r + c);
-        if (nvalid < kSmBK) {
-#pragma unroll
-          for (int c = 0; c < kSmBK; ++c)
-            if (c >= nvalid) r[c] = __float_as_uint(-INFINITY);
-        }
-        const float mt = a.scale_log2 * row_max<kSmBK>(r);
+        if (j == 0 && nt > 1) m2 = load_scores(o_col, 1);
+        const float mt = load_scores(s_col, j);
         if (j == 0) {
-          m2 = mt;
+          m2 = fmaxf(m2, mt);
         } else if (__any_sync(0xffffffffu, mt > m2 + kRescaleLog2)) {
           // warp-uniform (the TMEM accesses are .sync.aligned); O must hold PV(j-1)
           if (!(ok = mbar_wait_warp(smem_u32(o_done), (j - 1) & 1, abort_flag, a.status, 57))) break;

@@ -37,3 +37,30 @@ def test_small_attention(bsz, H, nq, nkv, dh, growing):
     err = np.linalg.norm(_f(o) - want) / np.linalg.norm(want)
     assert err < 1.5e-3, err
     assert B.sgd_kernel_status() == 0
+
+
+# Shapes of the dispatch rule's own table that go to the kernel of one query tile.
+@pytest.mark.parametrize("bsz,H,nq,nkv,dh", [(2, 20, 1024, 77, 64), (16, 16, 258, 258, 64), (2, 16, 136, 136, 72),
+                                             (1, 32, 333, 333, 128)])
+def test_first_reference_covers_128_keys(bsz, H, nq, nkv, dh):
+    """Probabilities are rounded to fp16 against the same reference as in the kernel of two query tiles
+    (impl 3), a row's maximum over its first 128 keys, so that the results agree but for the
+    order of the fp32 row sum: that moves a result by about 2^-22 before its rounding, across a
+    rounding boundary (2^-10 apart, relative) for one in 2^11 of them, by 2^-10.5 on average then:
+    2^-10.5 x sqrt(2^-11) = 1.6e-5 relative L2, allowed twice.  (A reference over 64 keys: 1.4e-4.)"""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2609_29505_gb300 import binding as B, build
+    build.build()
+    rng = np.random.default_rng(nq + nkv + dh)
+    hs = 80 if dh == 72 else dh
+    q, k, v = (torch.zeros(bsz, n, H, hs, dtype=torch.float16, device="cuda") for n in (nq, nkv, nkv))
+    for t in (q, k, v):
+        t[..., :dh] = _rand(rng, t.shape[:3] + (dh,)).cuda()
+    got = []
+    for impl in (0, 3):
+        o = torch.full((bsz, nq, H, dh), 7.0, dtype=torch.float16, device="cuda")
+        B.sgd_kernel_attention_hs(q, H * hs, k, v, H * hs, hs, o, H * dh, bsz, nq, nkv, H, dh, impl=impl)
+        got.append(_f(o).astype(np.float64))
+    assert np.linalg.norm(got[0] - got[1]) <= 3.2e-5 * np.linalg.norm(got[1])
+    assert B.sgd_kernel_status() == 0
