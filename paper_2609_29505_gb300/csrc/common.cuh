@@ -222,6 +222,18 @@ __device__ __forceinline__ void pdl_wait_and_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Four floats of what an earlier kernel of the step wrote (16-byte aligned).  A kernel of a step is
+// resident while its predecessor still writes, so that such data is not read-only for the kernel's
+// lifetime, as __ldg (ld.global.nc) demands: __ldg is for weights and tables alone.  As an
+// asm volatile the load stays behind pdl_wait_and_trigger but may pass stores to shared memory.
+__device__ __forceinline__ float4 ld_f32x4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+
 // ----------------------------------------------------------------------------
 // mbarrier
 // ----------------------------------------------------------------------------

@@ -95,8 +95,8 @@ __device__ __forceinline__ Affine4<MODE> load_affine4(const NormParams& p, int i
     if (p.b) a.b = __ldg(reinterpret_cast<const uint2*>(p.b + 4 * i));
   }
   if constexpr (MODE == kMod) {
-    a.sc = __ldg(reinterpret_cast<const float4*>(sc + 4 * i));
-    a.sh = __ldg(reinterpret_cast<const float4*>(sh + 4 * i));
+    a.sc = ld_f32x4(sc + 4 * i);
+    a.sh = ld_f32x4(sh + 4 * i);
   }
   if constexpr (MODE == kAny) {
     if (sc) {
@@ -589,7 +589,7 @@ __global__ void stem_patch_any_kernel(const StemParams p) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = 0.f;
     for (int k8 = 0; k8 < w_ld; ++k8) {
-      const float4 za = __ldg(z + 2 * k8), zb = __ldg(z + 2 * k8 + 1);
+      const float4 za = z[2 * k8], zb = z[2 * k8 + 1];
       const float zf[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(256) gemv_kernel(const GemvParams p) {
         const int i = i0 + j * blockDim.x;
         if (i < n4) {
           const int r = i / k4, k = (i - r * k4) << 2;
-          v[j] = __ldg(reinterpret_cast<const float4*>(p.x + static_cast<int64_t>(r) * p.ldx + k));
+          v[j] = ld_f32x4(p.x + static_cast<int64_t>(r) * p.ldx + k);
         }
       }
 #pragma unroll
@@ -798,7 +798,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) gemv_stream_kernel(const Ge
   for (int i = threadIdx.x; i < 8 * k4; i += kStreamThreads) {
     const int r = i / k4, k = (i - r * k4) << 2;
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);  // rows past the last contribute nothing and are not stored
-    if (r < p.rows) x = __ldg(reinterpret_cast<const float4*>(p.x + static_cast<int64_t>(r) * p.ldx + k));
+    if (r < p.rows) x = ld_f32x4(p.x + static_cast<int64_t>(r) * p.ldx + k);
     if (p.in_silu) x = make_float4(silu_f(x.x), silu_f(x.y), silu_f(x.z), silu_f(x.w));
     *reinterpret_cast<float4*>(xs + r * K + ((k & 4) ? half : 0) + (k >> 3) * 4) = x;
   }
@@ -889,12 +889,12 @@ __global__ void __launch_bounds__(128, 3) head_small_kernel(const HeadParams p) 
   for (int q = 0; q < 2; ++q) {
     const int64_t r = min(r0 + q, rows - 1);  // past the last row: computed again, not stored
     const int b = static_cast<int>(r / p.n_tokens);
-    const float4* x = reinterpret_cast<const float4*>(p.h + r * p.ldx);
+    const float* x = p.h + r * p.ldx;
     float4* xs = x0 + q * nv;
     float s1 = 0.f, sq = 0.f;
 #pragma unroll 4
     for (int i = lane; i < nv; i += 32) {
-      const float4 v = __ldg(x + i);
+      const float4 v = ld_f32x4(x + 4 * i);
       xs[i] = v;
       s1 += (v.x + v.y) + (v.z + v.w);
     }
