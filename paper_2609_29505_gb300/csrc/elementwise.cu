@@ -514,7 +514,8 @@ __global__ void __launch_bounds__(128) stem_patch_kernel(const StemParams p) {
   __shared__ float4 zs[kPatchRows][DIN / 4];
   pdl_wait_and_trigger();
   const IoSlot* s = p.slot;
-  const int rows = p.batch * p.n_tokens, r0 = blockIdx.y * kPatchRows, nr = min(kPatchRows, rows - r0);
+  const int col_blocks = ((p.d >> 2) + 127) / 128;  // in grid.x with the rows, which may be millions
+  const int rows = p.batch * p.n_tokens, r0 = (blockIdx.x / col_blocks) * kPatchRows, nr = min(kPatchRows, rows - r0);
   const int n_in = p.n_tokens - p.n_prefix;
   for (int i = threadIdx.x; i < nr * (DIN / 4); i += blockDim.x) {
     const int k = i / (DIN / 4), r = r0 + k;
@@ -522,7 +523,7 @@ __global__ void __launch_bounds__(128) stem_patch_kernel(const StemParams p) {
     if (n >= 0)
       zs[k][i % (DIN / 4)] = reinterpret_cast<const float4*>(s->state)[(static_cast<int64_t>(b) * n_in + n) * (DIN / 4) + i % (DIN / 4)];
   }
-  const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  const int c0 = ((blockIdx.x % col_blocks) * blockDim.x + threadIdx.x) * 4;
   const bool active = c0 < p.d;
   float w[4][DIN];
   if (active) {
@@ -1123,7 +1124,7 @@ cudaError_t stem_launch(const StemParams& p, cudaStream_t s) {
     const int gy = std::max(1, std::min(rows, 16 * num_sms() / gx));
     return launch_k(stem_rows_kernel, dim3(gx, gy), dim3(128), 0, s, p);
   }
-  const dim3 grid((p.d / 4 + 127) / 128, (rows + kPatchRows - 1) / kPatchRows);
+  const dim3 grid(((p.d / 4 + 127) / 128) * ((rows + kPatchRows - 1) / kPatchRows));
   if (p.d_in == 8) return launch_k(stem_patch_kernel<8>, grid, dim3(128), 0, s, p);
   if (p.d_in == 16) return launch_k(stem_patch_kernel<16>, grid, dim3(128), 0, s, p);
   if (p.d_in % 8 == 0) {
