@@ -102,9 +102,9 @@ typedef enum {
 /* Use 64-element K-blocks (4 stages, 128-byte swizzle) in the tcgen05 GEMMs. */
 #define SGD_FLAG_GEMM_BK64 8
 /* Launch a step's kernels with programmatic dependent launch: each kernel's launch and
- * prologue overlap the previous kernel's tail.  Every context does so (measured on GB300: tiny
- * -7%, DiT, U-ViT and SDXL-shaped -2 to -3%, LLaDA-8B-shaped -1% of the step's time; results are
- * the same bit for bit), so the flag is accepted and changes nothing. */
+ * prologue overlap the previous kernel's tail.  A context does so unless SGD_FLAG_SERIAL is set
+ * (measured on GB300: tiny -7%, DiT, U-ViT and SDXL-shaped -2 to -3%, LLaDA-8B-shaped -1% of the
+ * step's time; results are the same bit for bit), so this flag is accepted and changes nothing. */
 #define SGD_FLAG_PDL 16
 /* Fold RMSNorm / LayerNorm pre-norms into the GEMMs that follow them (Algorithm 2's
  * Norm -> projection as one tcgen05 GEMM: the gain folded into the weight, the row
@@ -113,6 +113,8 @@ typedef enum {
  * on GB300 it is slower (LLaDA-8B-shaped step -2% under the power cap, U-ViT / SDXL-shaped
  * -7 to -8%); results agree with the default path within fp16 rounding. */
 #define SGD_FLAG_FOLD_NORM 32
+/* Launch a step's kernels one after another instead: each starts when the one before has ended. */
+#define SGD_FLAG_SERIAL 64
 
 typedef struct {
   int stem, block, norm, mlp, head;   /* enums above                                   */

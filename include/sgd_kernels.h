@@ -95,6 +95,10 @@ typedef struct {
   float* stat_final;
 } sgd_epilogue_args;
 
+/* Kernel launches the calling thread has made so far with programmatic dependent launch (steps
+ * launched op by op, and the capture of their graphs in sgd_set_schedule). */
+SGD_API int sgd_kernel_dependent_launches(int64_t* launches);
+
 /* Partial-sum slots a residual writer with these arguments fills (see h16 above). */
 SGD_API int sgd_kernel_gemm_stat_slots(int M, int N, int K, const sgd_epilogue_args* epi,
                                        int variant, int* slots);

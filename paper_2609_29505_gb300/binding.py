@@ -42,6 +42,7 @@ FLAG_MMA_SYNC_ATTENTION = 2
 FLAG_GEMM_BK64 = 8
 FLAG_PDL = 16
 FLAG_FOLD_NORM = 32
+FLAG_SERIAL = 64
 
 EPI_F16, EPI_F32, EPI_DELTA, EPI_GATED, EPI_GELU, EPI_ROPE = range(6)
 KERNEL_NAMES = ["gemm_tc", "gemm_simt", "attention", "norm", "frozen_run", "small"]
@@ -54,7 +55,7 @@ EXPORTED = [
     "sgd_kernel_attention", "sgd_kernel_norm", "sgd_kernel_frozen_run", "sgd_kernel_status",
     "sgd_set_exec_mode", "sgd_step_host_async", "sgd_host_wait", "sgd_kernel_gemm_static_ws",
     "sgd_set_policy", "sgd_get_drift", "sgd_selftest_wait_timeout", "sgd_kernel_f16_clamped",
-    "sgd_kernel_gemm_stat_slots", "sgd_kernel_attention_hs",
+    "sgd_kernel_gemm_stat_slots", "sgd_kernel_attention_hs", "sgd_kernel_dependent_launches",
 ]
 EXEC_JAGGED_GRAPH, EXEC_EAGER, EXEC_PADDED_GRAPH = 0, 1, 2
 POLICY_STATIC, POLICY_DRIFT = 0, 1
@@ -147,6 +148,7 @@ def lib() -> C.CDLL:
             "sgd_kernel_status": (i, [C.POINTER(C.c_int)]),
             "sgd_kernel_f16_clamped": (i, [C.POINTER(C.c_int)]),
             "sgd_kernel_gemm_stat_slots": (i, [i, i, i, C.POINTER(sgd_epilogue_args), i, C.POINTER(C.c_int)]),
+            "sgd_kernel_dependent_launches": (i, [C.POINTER(i64)]),
             "sgd_set_exec_mode": (i, [vp, i]),
             "sgd_step_host_async": (i, [vp, vp, vp, f, vp, vp, i, vp]),
             "sgd_host_wait": (i, [vp]),
@@ -248,6 +250,12 @@ def sgd_kernel_status() -> int:
     st = C.c_int(0)
     check(lib().sgd_kernel_status(C.byref(st)), "sgd_kernel_status")
     return int(st.value)
+
+
+def sgd_kernel_dependent_launches() -> int:
+    n = C.c_int64(0)
+    check(lib().sgd_kernel_dependent_launches(C.byref(n)), "sgd_kernel_dependent_launches")
+    return int(n.value)
 
 
 def sgd_kernel_gemm_stat_slots(M, N, K, epi: "sgd_epilogue_args", variant=0) -> int:

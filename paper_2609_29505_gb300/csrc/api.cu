@@ -48,6 +48,11 @@ bool& pdl_flag() {
   return on;
 }
 
+int64_t& pdl_launches() {
+  thread_local int64_t n = 0;
+  return n;
+}
+
 }  // namespace sgd
 
 namespace {
@@ -813,7 +818,8 @@ int ensure_sk_ws(sgd_ctx* c) {
 
 // Launch a program's ops in order on `s`; with `pdl`, each kernel may begin launching while
 // the one before finishes (programmatic dependent launch; every kernel waits for its
-// predecessor's results before touching global memory).
+// predecessor's results before touching global memory, but for a GEMM's weight, which no kernel
+// of a step writes).
 int run_ops(const std::vector<Op>& ops, cudaStream_t s, bool pdl) {
   struct Scope {
     bool prev;
@@ -1175,7 +1181,7 @@ int sgd_create(const sgd_model_desc* desc, const sgd_weights* w, sgd_ctx** out) 
   if (!desc || !w || !out) return fail(SGD_ERR_ARG, "null argument");
   *out = nullptr;
   if (desc->flags & ~(SGD_FLAG_SIMT_GEMM | SGD_FLAG_MMA_SYNC_ATTENTION | SGD_FLAG_GEMM_BK64 | SGD_FLAG_PDL |
-                      SGD_FLAG_FOLD_NORM))
+                      SGD_FLAG_FOLD_NORM | SGD_FLAG_SERIAL))
     return fail(SGD_ERR_ARG, "unknown flag bits");
   int rc = check_shape(*desc, *w);
   if (rc) return rc;
@@ -1196,8 +1202,8 @@ int sgd_create(const sgd_model_desc* desc, const sgd_weights* w, sgd_ctx** out) 
   // A step is 20 to 200 kernels of 4 to 30 us (mid-size models), and the gap between two of them
   // was ~2 us: with each kernel's launch and prologue inside its predecessor's tail the steps of
   // the tiny / DiT / U-ViT / SDXL-shaped models take 672 / 5815 / 1627 / 617 us instead of 724 / 6000 /
-  // 1655 / 638 (whole short trajectories), the LLaDA-shaped blocks 8350 instead of 8430.
-  c->pdl = true;
+  // 1655 / 638 (whole short trajectories), the LLaDA-shaped blocks (under the power cap) 1% less.
+  c->pdl = (desc->flags & SGD_FLAG_SERIAL) == 0;
   // RMSNorm / LayerNorm pre-norms fold into the GEMMs that follow them on request; the AdaLN
   // modulation (a per-sample scale of the weight's columns) and the SIMT debug GEMM do not
   c->fold = (desc->norm == SGD_NORM_RMS || desc->norm == SGD_NORM_LN) &&
@@ -1926,6 +1932,12 @@ int sgd_selftest_wait_timeout(void* stream) {
   int* p = device_status_ptr();
   if (!p) return fail(SGD_ERR_CUDA, "status word unavailable");
   CUDA_TRY(wait_selftest_launch(p, SGD_SELFTEST_TIMEOUT_CODE, static_cast<cudaStream_t>(stream)));
+  return SGD_OK;
+}
+
+int sgd_kernel_dependent_launches(int64_t* launches) {
+  if (!launches) return fail(SGD_ERR_ARG, "null argument");
+  *launches = pdl_launches();
   return SGD_OK;
 }
 

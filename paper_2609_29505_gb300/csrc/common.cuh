@@ -681,6 +681,7 @@ static const int g_f16_clamp_registered = register_f16_clamp_flag(&f16_clamp_fla
 // api.cu) carry the programmatic-stream-serialization attribute, so that in a captured graph
 // each kernel's launch and prologue overlap the tail of the one before (programmatic edges).
 bool& pdl_flag();
+int64_t& pdl_launches();  // the calling thread's launches with the attribute
 
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
@@ -696,6 +697,7 @@ static inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 blo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    ++pdl_launches();
   }
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }

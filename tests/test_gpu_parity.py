@@ -329,16 +329,18 @@ def test_long_context_4096_tokens(B):
     m.close()
 
 
-@pytest.mark.parametrize("name", ["dit_small", "llada_small", "uvit_small", "sdxl_small"])
-def test_programmatic_dependent_launch_is_bit_identical(B, name):
-    """Step programs launched with programmatic dependent launch (SGD_FLAG_PDL: each kernel's
+@pytest.mark.parametrize("fold", [False, True])
+@pytest.mark.parametrize("name", SMALL)
+def test_programmatic_dependent_launch_is_bit_identical(B, name, fold):
+    """Step programs launched with programmatic dependent launch (the default: each kernel's
     launch and prologue overlapping its predecessor's tail, in graphs and eagerly) give the
-    same bits as fully serialised launches."""
+    same bits as serialised launches (SGD_FLAG_SERIAL), in which no kernel carries the attribute."""
     c = case(name, 0.5)
     results = []
-    for flags, mode in ((0, B.EXEC_JAGGED_GRAPH), (B.FLAG_PDL, B.EXEC_JAGGED_GRAPH),
-                        (B.FLAG_PDL, B.EXEC_EAGER)):
-        m = B.Denoiser(c.cfg, c.w_dev, flags=flags)
+    for serial, mode in ((True, B.EXEC_JAGGED_GRAPH), (True, B.EXEC_EAGER), (False, B.EXEC_JAGGED_GRAPH),
+                         (False, B.EXEC_EAGER)):
+        n0 = B.sgd_kernel_dependent_launches()
+        m = B.Denoiser(c.cfg, c.w_dev, flags=(B.FLAG_SERIAL if serial else 0) | (B.FLAG_FOLD_NORM if fold else 0))
         m.set_schedule(c.T, c.sched["lifetimes"], c.sched["groups"])
         m.set_exec_mode(mode)
         out = c.out_buffer()
@@ -349,6 +351,7 @@ def test_programmatic_dependent_launch_is_bit_identical(B, name):
             res.append(out.cpu().clone())
         m.check_device()
         m.close()
+        assert (B.sgd_kernel_dependent_launches() == n0) == serial
         results.append(res)
     for other in results[1:]:
         for a, b in zip(results[0], other):
