@@ -99,6 +99,12 @@ typedef struct {
  * launched op by op, and the capture of their graphs in sgd_set_schedule). */
 SGD_API int sgd_kernel_dependent_launches(int64_t* launches);
 
+/* The tile sgd_kernel_gemm takes for these arguments on the current device: CTAs of a group per tile
+ * (1 or 2; 0: the one-CTA kernel of the forced forms and folded norms, or the SIMT kernel) and
+ * the tile's columns of B. */
+SGD_API int sgd_kernel_gemm_tile(int M, int N, int K, const sgd_epilogue_args* epi, int variant,
+                                 int* group, int* columns);
+
 /* Partial-sum slots a residual writer with these arguments fills (see h16 above). */
 SGD_API int sgd_kernel_gemm_stat_slots(int M, int N, int K, const sgd_epilogue_args* epi,
                                        int variant, int* slots);

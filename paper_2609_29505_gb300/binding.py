@@ -55,7 +55,7 @@ EXPORTED = [
     "sgd_kernel_attention", "sgd_kernel_norm", "sgd_kernel_frozen_run", "sgd_kernel_status",
     "sgd_set_exec_mode", "sgd_step_host_async", "sgd_host_wait", "sgd_kernel_gemm_static_ws",
     "sgd_set_policy", "sgd_get_drift", "sgd_selftest_wait_timeout", "sgd_kernel_f16_clamped",
-    "sgd_kernel_gemm_stat_slots", "sgd_kernel_attention_hs", "sgd_kernel_dependent_launches",
+    "sgd_kernel_gemm_stat_slots", "sgd_kernel_attention_hs", "sgd_kernel_dependent_launches", "sgd_kernel_gemm_tile",
 ]
 EXEC_JAGGED_GRAPH, EXEC_EAGER, EXEC_PADDED_GRAPH = 0, 1, 2
 POLICY_STATIC, POLICY_DRIFT = 0, 1
@@ -148,6 +148,8 @@ def lib() -> C.CDLL:
             "sgd_kernel_status": (i, [C.POINTER(C.c_int)]),
             "sgd_kernel_f16_clamped": (i, [C.POINTER(C.c_int)]),
             "sgd_kernel_gemm_stat_slots": (i, [i, i, i, C.POINTER(sgd_epilogue_args), i, C.POINTER(C.c_int)]),
+            "sgd_kernel_gemm_tile": (i, [i, i, i, C.POINTER(sgd_epilogue_args), i, C.POINTER(C.c_int),
+                                         C.POINTER(C.c_int)]),
             "sgd_kernel_dependent_launches": (i, [C.POINTER(i64)]),
             "sgd_set_exec_mode": (i, [vp, i]),
             "sgd_step_host_async": (i, [vp, vp, vp, f, vp, vp, i, vp]),
@@ -256,6 +258,13 @@ def sgd_kernel_dependent_launches() -> int:
     n = C.c_int64(0)
     check(lib().sgd_kernel_dependent_launches(C.byref(n)), "sgd_kernel_dependent_launches")
     return int(n.value)
+
+
+def sgd_kernel_gemm_tile(M, N, K, epi: "sgd_epilogue_args", variant=0):
+    group, columns = C.c_int(0), C.c_int(0)
+    check(lib().sgd_kernel_gemm_tile(M, N, K, C.byref(epi), int(variant), C.byref(group), C.byref(columns)),
+          "sgd_kernel_gemm_tile")
+    return int(group.value), int(columns.value)
 
 
 def sgd_kernel_gemm_stat_slots(M, N, K, epi: "sgd_epilogue_args", variant=0) -> int:

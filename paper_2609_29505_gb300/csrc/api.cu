@@ -1756,7 +1756,7 @@ int kernel_ws(int dev, void* stream, size_t floats, int n_cnt, KernelWs** out) {
 // The kernel-level GEMM arguments as a validated plan (variant codes: sgd_kernel_gemm);
 // returns an sgd_status.  Nothing touches the device before the checks pass.
 int kernel_gemm_plan(const void* A, int lda, const void* B, int ldb, int M, int N, int K,
-                     const sgd_epilogue_args* ea, int variant, GemmPlan& p) {
+                     const sgd_epilogue_args* ea, int variant, GemmPlan& p, bool allow_group = true) {
   if (!ea) return fail(SGD_ERR_ARG, "null epilogue");
   if (ea->kind < 0 || ea->kind > SGD_EPI_ROPE) return fail(SGD_ERR_ARG, "bad epilogue kind");
   if (variant < 0 || variant > 12 || variant == 2 || variant == 4)
@@ -1769,7 +1769,7 @@ int kernel_gemm_plan(const void* A, int lda, const void* B, int ldb, int M, int 
   p.N = N;
   p.K = K;
   p.simt = variant == 1;
-  p.allow_group = p.encode && variant == 0;  // (the statistics slots are those of the one-CTA kernel)
+  p.allow_group = allow_group && variant == 0;
   p.bk = variant == 3 ? 32 : 64;
   if (variant == 5) { p.bn = 256; p.epiw = 4; }
   if (variant == 6) { p.bn = 256; p.epiw = 8; }
@@ -1817,6 +1817,13 @@ int kernel_gemm_plan(const void* A, int lda, const void* B, int ldb, int M, int 
   const int rc = gemm_plan(p, &why);
   if (rc) return fail(rc == -5 ? SGD_ERR_CUDA : (rc == -1 ? SGD_ERR_ARG : SGD_ERR_SHAPE), why);
   return SGD_OK;
+}
+
+// The plan's tile alone: chosen on the host from the shape, so planned with dummy aligned operands.
+int plan_tile(int M, int N, int K, const sgd_epilogue_args* ea, int variant, bool allow_group, GemmPlan& p) {
+  static const uint4 dummy[1] = {};
+  p.encode = false;
+  return kernel_gemm_plan(dummy, K, dummy, K, M, N, K, ea, variant, p, allow_group);
 }
 
 }  // namespace
@@ -1941,14 +1948,20 @@ int sgd_kernel_dependent_launches(int64_t* launches) {
   return SGD_OK;
 }
 
+int sgd_kernel_gemm_tile(int M, int N, int K, const sgd_epilogue_args* ea, int variant, int* group, int* columns) {
+  if (!group || !columns || !ea) return fail(SGD_ERR_ARG, "null argument");
+  GemmPlan p;
+  const int rc = plan_tile(M, N, K, ea, variant, true, p);
+  if (rc) return rc;
+  *group = p.group;
+  *columns = p.simt ? 0 : p.bn;
+  return SGD_OK;
+}
+
 int sgd_kernel_gemm_stat_slots(int M, int N, int K, const sgd_epilogue_args* ea, int variant, int* slots) {
   if (!slots || !ea) return fail(SGD_ERR_ARG, "null argument");
-  // the tile width is chosen on the host from the shape alone; plan with dummy aligned operands
-  static const uint4 dummy[1] = {};
-  sgd_epilogue_args e = *ea;
   GemmPlan p;
-  p.encode = false;
-  int rc = kernel_gemm_plan(dummy, K, dummy, K, M, N, K, &e, variant, p);
+  const int rc = plan_tile(M, N, K, ea, variant, false, p);  // statistics are written by the one-CTA kernel
   if (rc) return rc;
   *slots = p.simt ? 0 : 2 * ((N + p.bn - 1) / p.bn);
   return SGD_OK;
