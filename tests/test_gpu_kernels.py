@@ -557,3 +557,57 @@ def test_attention_dh72_head_padded(B, H, nq, nkv, bsz, impl):
     assert err < 1.5e-3, err
     assert np.max(np.abs(got - want)) < 5e-3 * float(np.abs(want).max())
     assert B.sgd_kernel_status() == 0
+
+
+# rows: fewer and more than one wave of blocks where a row has its own block (8 blocks an SM: 1216).
+# mod: none; 16-byte aligned; at an odd float's address with an odd row stride.
+@pytest.mark.parametrize("rows,d", [(5, 256), (131, 1152), (131, 1284), (131, 2052), (1301, 2052), (1301, 4096)])
+@pytest.mark.parametrize("affine", ["none", "gain", "gain_shift"])
+@pytest.mark.parametrize("mod", ["none", "aligned", "odd"])
+def test_norm_forms(B, rows, d, affine, mod):
+    """Every combination of gain, shift and modulation, in one warp per row, one block per row and
+    blocks that walk over the rows."""
+    rng = np.random.default_rng(rows + d)
+    rpb = 100
+    kind = 0 if affine == "gain" else (1 if affine == "gain_shift" else 2)
+    h = torch.from_numpy((rng.standard_normal((rows, d)) * 3 + 0.5).astype(np.float32)).cuda()
+    g = _rand(rng, (d,), 0.1).float().add(1.0).to(torch.bfloat16).cuda() if affine != "none" else None
+    b = _rand(rng, (d,), 0.1, torch.bfloat16).cuda() if affine == "gain_shift" else None
+    out = torch.full((rows, d), 7.0, dtype=torch.float16, device="cuda")
+    kw = {}
+    if mod != "none":
+        n, ld, at = -(-rows // rpb), 2 * d + (mod == "odd"), int(mod == "odd")
+        buf = torch.from_numpy((0.3 * rng.standard_normal(n * ld + at + 8)).astype(np.float32)).cuda()
+        shift, scale = (torch.as_strided(buf, (n, d), (ld, 1), at + o) for o in (0, d))
+        kw = dict(shift=shift, scale=scale, ld_mod=ld, rows_per_batch=rpb)
+    B.sgd_kernel_norm(h, out, rows, d, kind, g=g, b=b, eps=1e-6, **kw)
+    torch.cuda.synchronize()
+    hn = h.cpu().numpy()
+    if kind == 0:
+        want = odn.rms_norm(hn, _f(g), 1e-6)
+    else:
+        want = odn.layer_norm(hn, None if g is None else _f(g), None if b is None else _f(b), 1e-6)
+    if mod != "none":
+        smp = np.arange(rows) // rpb
+        want = want * (1 + _f(scale)[smp]) + _f(shift)[smp]
+    _check_f16(out, want, extra_abs=1e-5)
+
+
+@pytest.mark.parametrize("n", [1, 7, 4096, 100003])
+@pytest.mark.parametrize("at_z,at_e", [(0, 0), (1, 0), (0, 3), (2, 2)])
+def test_sampler_at_any_address(B, n, at_z, at_e):
+    """z <- alpha z - beta eps at 16-byte and other addresses, in place; nothing around it written."""
+    rng = np.random.default_rng(n)
+    z0, e0 = (rng.standard_normal(n + 8).astype(np.float32) for _ in range(2))
+    z, e = torch.from_numpy(z0.copy()).cuda(), torch.from_numpy(e0).cuda()
+    B.sgd_sampler_update(z[at_z:at_z + n], e[at_e:at_e + n], 0.9, 0.2)
+    torch.cuda.synchronize()
+    want = z0.copy()
+    a, b = np.float32(0.9), np.float32(0.2)
+    want[at_z:at_z + n] = a * z0[at_z:at_z + n] - b * e0[at_e:at_e + n]
+    # one rounding more or less per product: 2^-23 of |alpha z| + |beta eps|
+    bound = 2.0 ** -23 * (np.abs(a * z0[at_z:at_z + n]) + np.abs(b * e0[at_e:at_e + n]))
+    got = z.cpu().numpy()
+    assert (np.abs(got[at_z:at_z + n] - want[at_z:at_z + n]) <= bound).all()
+    got[at_z:at_z + n] = want[at_z:at_z + n]
+    np.testing.assert_array_equal(got, want)

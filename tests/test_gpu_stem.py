@@ -35,3 +35,13 @@ def test_more_token_rows_than_a_grid_dimension_holds():
                                                batch=2048, n_tokens=258, T=1, horizons=[1])
     got, want = _step(cfg, [0, 1, 1024, 2047])
     assert np.linalg.norm(got - want) <= 5e-3 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("d_in", [8, 16, 24, 12])
+def test_patch_widths(d_in):
+    """Weight rows in registers (8, 16 channels), read as vectors (24) and one by one (12); 201 token rows
+    end inside a block's 8, and 576 channels inside the second block's 512."""
+    cfg = synth.get_config("uvit_small").with_(name="uvit_patch%d" % d_in, n_blocks=1, n_skips=0, d=576, n_heads=9,
+                                               d_ff=128, n_tokens=67, d_in=d_in, T=1, horizons=[1])
+    got, want = _step(cfg, [0, 1, 2])
+    assert np.linalg.norm(got - want) <= 5e-3 * np.linalg.norm(want)
