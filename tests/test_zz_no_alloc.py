@@ -125,6 +125,28 @@ def test_static_ws_rejects_a_split_larger_than_its_scratch(B):
     assert B.sgd_kernel_status() == 0
 
 
+@pytest.mark.gpu
+def test_static_ws_keeps_its_size_limit_where_it_picks_the_kernel(B):
+    """Variant 0 keeps the entry's limit, that of the one-CTA kernel's split, whichever kernel it runs:
+    1792 x 4608 x 4096 leaves 100 of 252 tiles (152 SMs) in 3 segments, 37.5 MiB.  The allocating
+    entry runs it."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("a size for 152 SMs")
+    M, N, K = 1792, 4608, 4096
+    A, W, h0 = _problem(M, N, K, "f16", 13)
+    out = torch.full((M, N), 7.0, dtype=torch.float16, device="cuda")
+    e = B.sgd_epilogue_args(kind=B.EPI_F16, out=out.data_ptr(), ldo=N)
+    with pytest.raises(B.SgdError) as err:
+        B.sgd_kernel_gemm_static_ws(A, W, M, N, K, e, 0)
+    assert err.value.code == B.SGD_ERR_SHAPE
+    torch.cuda.synchronize()
+    assert bool((out == 7.0).all())
+    B.sgd_kernel_gemm(A, W, M, N, K, e)
+    torch.cuda.synchronize()
+    assert not bool((out == 7.0).all())
+    assert B.sgd_kernel_status() == 0
+
+
 def test_static_ws_validates_on_host():
     """Argument errors are reported before the device is touched (runs without a GPU)."""
     from paper_2609_29505_gb300 import build
