@@ -1273,23 +1273,27 @@ int attn_check(const AttnParams& p, const char** why) {
   return 0;
 }
 
-// Whether attn_sm_kernel runs this shape faster than attn_pp_kernel, by the time of each in us:
-// a pair CTA holds an SM for a fixed part and ~1.2 us per 128 keys; a CTA of attn_sm_kernel takes
-// ~1 us per 64 keys by itself, and the SM ~0.5 us (d_h 64; 0.6, 0.8) for one of several.  Fitted to
-// 22 shapes (measured us, pair / this kernel):
-//   16 x 258 tokens, 16 heads of 64    27.0 / 17.3     2 x 1024, 20 heads of 64         26.4 / 22.1
-//   2 x 1024 x 77 keys, 20 heads of 64 10.9 /  7.0     4 x 512, 16 heads of 64           9.4 / 11.3
-//   1 x 333, 32 heads of 128           10.3 /  9.9     4 x 1024, 32 heads of 128        76.6 / 90.3
-//   8 x 256, 16 heads of 72             8.3 /  8.8     2 x 136, 16 heads of 72           7.8 /  6.4
+// Whether attn_sm_kernel runs this shape faster than attn_pp_kernel, by the time of each in us: a
+// pair CTA holds an SM for a fixed part (more where it has both query tiles) and 1.1 to 1.4 us per
+// 128 keys; a CTA of attn_sm_kernel takes a fixed part (more where the first reference looks at a
+// second key tile) and 0.8 to 1 us per 64 keys by itself, and the SM 0.5 (d_h 64), 0.6 or 0.8 for one
+// of several.  Fitted to 28 shapes, of which the chosen kernel is within 8% of the better one
+// (measured us, pair / this kernel):
+//   16 x 258 tokens, 16 heads of 64    24.9 / 17.3     2 x 1024, 20 heads of 64         24.2 / 20.6
+//   2 x 1024 x 77 keys, 20 heads of 64 10.1 /  7.0     4 x 512, 16 heads of 64           8.6 / 11.2
+//   1 x 333, 32 heads of 128            9.2 /  9.9     4 x 1024, 32 heads of 128        67.0 / 91.5
+//   8 x 256, 16 heads of 72             7.8 /  8.7     2 x 136, 16 heads of 72           7.1 /  6.6
+//   10 x 97 x 200 keys, 16 heads of 128 11.8 / 9.8     1 x 128, 8 heads of 64            4.3 /  4.8
 bool attn_small(const AttnParams& p) {
   const double sms = num_sms(), heads = static_cast<double>(p.batch) * p.n_heads;
   const double pairs = std::ceil(p.n_q / 256.0) * heads, ctas = std::ceil(p.n_q / 128.0) * heads;
   const double nt = std::ceil(p.n_kv / 128.0), nt64 = std::ceil(p.n_kv / 64.0);
-  const bool d64 = p.d_head == 64, d72 = p.d_head == 72;
-  const double pair_fixed = p.d_head == 128 ? 5.0 : 3.0, pair_tile = d64 ? 1.14 : (d72 ? 1.3 : 1.15);
+  const bool d64 = p.d_head == 64, d72 = p.d_head == 72, d128 = p.d_head == 128, two = p.n_q > kTcBQ;
+  const double pair_fixed = d128 ? (two ? 4.9 : 4.5) : (two ? 3.8 : 3.0), pair_tile = d64 ? 1.14 : (d72 ? 1.3 : 1.42);
+  const double sm_fixed = (d128 ? 4.0 : 2.0) + (nt64 > 1 ? 0.6 : 0.0), one_tile = d128 ? 0.83 : 1.0;
   const double sm_tile = d64 ? 0.52 : (d72 ? 0.6 : 0.8), slots = sms * (d64 ? 3 : 2);
   const double t_pair = std::ceil(pairs / sms) * (pair_fixed + nt * pair_tile);
-  const double t_small = 2.0 + nt64 * std::max(std::ceil(ctas / slots), sm_tile * ctas / sms);
+  const double t_small = sm_fixed + nt64 * std::max(one_tile * std::ceil(ctas / slots), sm_tile * ctas / sms);
   return t_small < t_pair;
 }
 
