@@ -139,10 +139,12 @@ __device__ __forceinline__ float4 norm_apply4(const NormParams& p, const Affine4
 // Rows wider than 2048 (LLaDA's 4096): 256 threads per row, kWideVec float4 each, and a grid of
 // a few blocks per SM that walk over the rows with the next row's loads in flight while the
 // current one is reduced and stored.  One block per row left the loads of a block's only row
-// exposed and a second, two-thirds full wave (4096 x 4096: 23.6 us against 19.2; bound by HBM).
+// exposed and a second, two-thirds full wave: 4096 x 4096 with h from DRAM 23.8 us, 18.7 so (5.4 of
+// the 6.7 TB/s of a copy: one row ahead per block, with a barrier between its loads and its stores,
+// is too little in flight); with h still in L2 17.0 and 15.9.
 // Rows that fit in one wave of blocks get a block of 128 threads each (kPipe false).
 constexpr int wide_threads(bool pipe) { return pipe ? 256 : 128; }  // d <= 4096: 4 or 8 float4 per thread
-// per SM (with a gain alone the pipelined rows fit four blocks: 19.4 -> 18.8 us at 4096 x 4096)
+// per SM (with a gain alone the pipelined rows fit four blocks: 3% faster than three at 4096 x 4096)
 constexpr int wide_blocks(int mode, bool pipe) { return pipe ? (mode == kGain ? 4 : 3) : 8; }
 template <int MODE, bool kPipe>
 __global__ void __launch_bounds__(wide_threads(kPipe), wide_blocks(MODE, kPipe)) norm_wide_kernel(const NormParams p) {

@@ -1,7 +1,7 @@
 // Host side of the tcgen05 GEMM (planning: tile shape, tile order, stream-K split, tensor
 // maps; dispatch to the kernel instantiations), the SIMT reference GEMM, the device status
-// word and the fixed scratch of the allocation-free entry.  The kernel itself is in
-// gemm_kernel.cuh.
+// word and the fixed scratch of the allocation-free entry.  The kernels themselves are in
+// gemm_group_kernel.cuh (the default) and gemm_kernel.cuh (folded norms and the forced forms).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -487,7 +487,6 @@ int gemm_plan(GemmPlan& p, const char** why) {
 size_t gemm_ws_floats(const GemmPlan& p) {
   return p.sk_tiles > 0 ? static_cast<size_t>(p.sk_tiles) * p.max_seg * kBM * p.bn : 0;
 }
-
 
 template <int FEAT>
 cudaError_t launch_feat(const GemmPlan& p, const TcArgs& a, cudaStream_t s) {

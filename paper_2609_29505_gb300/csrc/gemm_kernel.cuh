@@ -1071,7 +1071,7 @@ __global__ void __launch_bounds__(TileCfg<BK, BN, EPIW>::kThreads, 1)
       const bool ok = warp_wait(&tfull[acc], aph, abort_flag, a.status, 4);
       if (k0 == 0 && k1 == a.num_k) {  // the whole K range of the tile lies in this CTA's share
         if (ok) {
-            tc_fence_after();
+          tc_fence_after();
           epilogue_tile<kBN, kEpiWarps == 4, FEAT>(a, out, row, n_blk, TmemSrc{tbase, a.epi.alpha}, cb, ce, part,
                                            kEpiWarps == 8 ? 2 : 1, stg);
           tc_fence_before();
